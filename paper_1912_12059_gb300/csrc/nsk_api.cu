@@ -7,6 +7,8 @@
 #include <string.h>
 
 #include <atomic>
+#include <cmath>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -20,15 +22,16 @@ namespace {
 // ---- nodal basis (Sec. 3.1): Gauss-Legendre / Gauss-Lobatto nodes and weights ----
 
 // P_n(x) and P_{n-1}(x) by the Bonnet recurrence.
-void legendre_pair(int n, double x, double* pn, double* pnm1) {
-  double a = 1.0, b = x;  // P_0, P_1
+template <typename T>
+void legendre_pair(int n, T x, T* pn, T* pnm1) {
+  T a = 1.0, b = x;  // P_0, P_1
   if (n == 0) {
     *pn = 1.0;
     *pnm1 = 0.0;
     return;
   }
   for (int k = 2; k <= n; ++k) {
-    const double c = ((2 * k - 1) * x * b - (k - 1) * a) / k;
+    const T c = ((2 * k - 1) * x * b - (k - 1) * a) / k;
     a = b;
     b = c;
   }
@@ -38,20 +41,21 @@ void legendre_pair(int n, double x, double* pn, double* pnm1) {
 
 // Gauss-Legendre: the n = N+1 roots of P_n, Newton from Tricomi's estimate;
 // weights 2 (1 - x^2) / (n P_{n-1}(x))^2.
-void gauss_legendre(int n, double* x, double* w) {
+template <typename T>
+void gauss_legendre(int n, T* x, T* w) {
   const double pi = 3.141592653589793238462643;
   for (int i = 0; i < n; ++i) {
     const double theta = pi * (4.0 * (n - i) - 1.0) / (4.0 * n + 2.0);
-    double z = (1.0 - 1.0 / (8.0 * n * n) + 1.0 / (8.0 * n * n * n)) * cos(theta);
+    T z = (1.0 - 1.0 / (8.0 * n * n) + 1.0 / (8.0 * n * n * n)) * cos(theta);
     for (int it = 0; it < 60; ++it) {
-      double pn, pm;
+      T pn, pm;
       legendre_pair(n, z, &pn, &pm);
-      const double dp = n * (pm - z * pn) / (1.0 - z * z);
-      const double dz = pn / dp;
+      const T dp = n * (pm - z * pn) / (1.0 - z * z);
+      const T dz = pn / dp;
       z -= dz;
-      if (fabs(dz) <= 1e-17) break;
+      if (std::fabs(dz) <= 1e-17) break;
     }
-    double pn, pm;
+    T pn, pm;
     legendre_pair(n, z, &pn, &pm);
     x[i] = z;
     w[i] = 2.0 * (1.0 - z * z) / ((n * pm) * (n * pm));
@@ -60,49 +64,59 @@ void gauss_legendre(int n, double* x, double* w) {
 
 // Gauss-Lobatto with N+1 nodes: +-1 and the roots of P_N'; Newton with
 // P_N'' from Legendre's differential equation; weights 2 / (N (N+1) P_N(x)^2).
-void gauss_lobatto(int N, double* x, double* w) {
+template <typename T>
+void gauss_lobatto(int N, T* x, T* w) {
   const double pi = 3.141592653589793238462643;
   x[0] = -1.0;
   x[N] = 1.0;
   for (int i = 1; i < N; ++i) {
-    double z = -cos(pi * i / N);
+    T z = -cos(pi * i / N);
     for (int it = 0; it < 60; ++it) {
-      double pn, pm;
+      T pn, pm;
       legendre_pair(N, z, &pn, &pm);
-      const double d1 = N * (pm - z * pn) / (1.0 - z * z);
-      const double d2 = (2.0 * z * d1 - N * (N + 1.0) * pn) / (1.0 - z * z);
-      const double dz = d1 / d2;
+      const T d1 = N * (pm - z * pn) / (1.0 - z * z);
+      const T d2 = (2.0 * z * d1 - N * (N + 1.0) * pn) / (1.0 - z * z);
+      const T dz = d1 / d2;
       z -= dz;
-      if (fabs(dz) <= 1e-17) break;
+      if (std::fabs(dz) <= 1e-17) break;
     }
     x[i] = z;
   }
   for (int i = 0; i <= N; ++i) {
-    double pn, pm;
+    T pn, pm;
     legendre_pair(N, x[i], &pn, &pm);
     w[i] = 2.0 / (N * (N + 1.0) * pn * pn);
   }
 }
 
 // Barycentric weights, derivative matrix D_ij = l_j'(x_i) and l_j(x0).
-void barycentric(int n, const double* x, double* lam) {
+template <typename T>
+void barycentric(int n, const T* x, T* lam) {
   for (int j = 0; j < n; ++j) {
-    double p = 1.0;
+    T p = 1.0;
     for (int m = 0; m < n; ++m)
       if (m != j) p *= x[j] - x[m];
     lam[j] = 1.0 / p;
   }
 }
-double lagrange_at(int n, const double* x, const double* lam, int j, double x0) {
+template <typename T>
+T lagrange_at(int n, const T* x, const T* lam, int j, T x0) {
   for (int m = 0; m < n; ++m)
     if (x0 == x[m]) return m == j ? 1.0 : 0.0;
-  double s = 0.0;
+  T s = 0.0;
   for (int m = 0; m < n; ++m) s += lam[m] / (x0 - x[m]);
   return lam[j] / (x0 - x[j]) / s;
 }
 
-template <typename R>
-void fill_tab(NskTab<R>& t, int n, const double* x, const double* w) {
+// The reference operator of a node set in FP64: dvol[i*NSK_MAXNP + j] = (w_j / w_i) l_i'(xi_j) the
+// weak-form volume operator, lm/lp[j] = l_j(-1) / l_j(+1) the prolongation to the faces, lmw/lpw[i] =
+// l_i(-1) / w_i, l_i(+1) / w_i the surface lifting.
+struct NskBasis {
+  double dvol[NSK_MAXNP * NSK_MAXNP];
+  double lm[NSK_MAXNP], lp[NSK_MAXNP], lmw[NSK_MAXNP], lpw[NSK_MAXNP];
+};
+NskBasis make_basis(int n, const double* x, const double* w) {
+  NskBasis t;
   double lam[NSK_MAXNP], D[NSK_MAXNP][NSK_MAXNP];
   barycentric(n, x, lam);
   for (int i = 0; i < n; ++i) {
@@ -116,14 +130,14 @@ void fill_tab(NskTab<R>& t, int n, const double* x, const double* w) {
   }
   memset(&t, 0, sizeof(t));
   for (int i = 0; i < n; ++i) {
-    for (int j = 0; j < n; ++j) t.dvol[i * NSK_MAXNP + j] = (R)(w[j] / w[i] * D[j][i]);
+    for (int j = 0; j < n; ++j) t.dvol[i * NSK_MAXNP + j] = w[j] / w[i] * D[j][i];
     const double lm = lagrange_at(n, x, lam, i, -1.0), lp = lagrange_at(n, x, lam, i, 1.0);
-    t.lm[i] = (R)lm;
-    t.lp[i] = (R)lp;
-    t.lmw[i] = (R)(lm / w[i]);
-    t.lpw[i] = (R)(lp / w[i]);
-    t.w[i] = (R)w[i];
+    t.lm[i] = lm;
+    t.lp[i] = lp;
+    t.lmw[i] = lm / w[i];
+    t.lpw[i] = lp / w[i];
   }
+  return t;
 }
 
 // Spinodal densities of the reduced VdW fluid: p'(rho) = 0 <=> rho (3 - rho)^2 = 4 T, one root
@@ -147,10 +161,14 @@ void spinodal_interval(double T, double* lo, double* hi) {
 
 // model coefficients of both operator precisions (after the mesh and the parameters are known)
 template <typename R>
-void fill_coef(NskTab<R>& t, const NskParams& p) {
-  const NskTab<double>& td = p.td;  // the FP64 operator tables (already filled)
+void fill_coef(NskTab<R>& t, const NskParams& p, const NskBasis& td, int n, const double* w) {
+  memset(&t, 0, sizeof(t));
+  for (int i = 0; i < n; ++i) t.w[i] = (R)w[i];
+  for (int i = 0; i < NSK_MAXNP; ++i) {
+    t.lm[i] = (R)td.lm[i];
+    t.lp[i] = (R)td.lp[i];
+  }
   for (int k = 0; k < 3; ++k) {
-    t.rh[k] = (R)p.rh[k];
     for (int i = 0; i < NSK_MAXNP; ++i) {
       for (int j = 0; j < NSK_MAXNP; ++j) t.dk[k][i * NSK_MAXNP + j] = (R)(p.rh[k] * td.dvol[i * NSK_MAXNP + j]);
       t.lpk[k][i] = (R)(p.rh[k] * td.lpw[i]);
@@ -169,6 +187,104 @@ void fill_coef(NskTab<R>& t, const NskParams& p) {
   t.ab = (R)(p.alpha / p.beta);
 }
 
+// The reference operator in extended precision as integers of 2^-56 (exact to 58 bits of a row's
+// sum, which the fixed-point tables of nsk_fx.cuh keep): row i the np volume entries
+// (w_j / w_i) l_i'(x_j), then -l_i(+1) / (2 w_i) and l_i(-1) / (2 w_i); l: l_j(-1), l_j(+1); and
+// the largest row sums. Formed once per node set and order.
+struct FxBase {
+  long long m[NSK_MAXNP][NSK_MAXNP + 2], l[2][NSK_MAXNP];
+  double msum, lsum;
+};
+void make_fx_base(FxBase& b, int node_type, int np) {
+  typedef long double T;
+  T x[NSK_MAXNP], w[NSK_MAXNP], lam[NSK_MAXNP], M[NSK_MAXNP][NSK_MAXNP + 2], l[2][NSK_MAXNP];
+  if (node_type == NSK_NODES_GAUSS)
+    gauss_legendre(np, x, w);
+  else
+    gauss_lobatto(np - 1, x, w);
+  barycentric(np, x, lam);
+  for (int i = 0; i < np; ++i) {
+    T diag = 0.0;
+    for (int j = 0; j < np; ++j) {
+      if (i == j) continue;
+      const T d = lam[j] / lam[i] / (x[i] - x[j]);  // l_j'(x_i)
+      M[j][i] = w[i] / w[j] * d;
+      diag -= d;
+    }
+    M[i][i] = diag;
+    l[0][i] = lagrange_at(np, x, lam, i, (T)-1.0);
+    l[1][i] = lagrange_at(np, x, lam, i, (T)1.0);
+    M[i][np] = (T)-0.5 * l[1][i] / w[i];
+    M[i][np + 1] = (T)0.5 * l[0][i] / w[i];
+  }
+  b.msum = b.lsum = 0.0;
+  for (int i = 0; i < np; ++i) {
+    double r = 0.0;
+    for (int j = 0; j < np + 2; ++j) {
+      b.m[i][j] = llrintl(ldexpl(M[i][j], 56));
+      r += std::fabs((double)M[i][j]);
+    }
+    b.msum = std::fmax(b.msum, r);
+  }
+  for (int s = 0; s < 2; ++s) {
+    double r = 0.0;
+    for (int j = 0; j < np; ++j) {
+      b.l[s][j] = llrintl(ldexpl(l[s][j], 56));
+      r += std::fabs((double)l[s][j]);
+    }
+    b.lsum = std::fmax(b.lsum, r);
+  }
+}
+const FxBase& fx_base(int node_type, int np) {
+  static FxBase base[2][NSK_MAXNP + 1];
+  static std::once_flag once[2][NSK_MAXNP + 1];
+  const int t = node_type == NSK_NODES_GAUSS ? 0 : 1;
+  std::call_once(once[t][np], [&] { make_fx_base(base[t][np], node_type, np); });
+  return base[t][np];
+}
+
+// biased exponent of a positive value (0: zero)
+int biased_exp(double x) {
+  int e = 0;
+  if (!(x > 0.0)) return 0;
+  frexp(x, &e);
+  return e + 1022 > 0 ? e + 1022 : 0;
+}
+// c m 2^-56 (m an entry of FxBase, c >= 0) in the two-limb form at the biased exponent es,
+// (h 2^28 + l) 2^(es - 1023 - 57), rounded
+int2 fx_entry(long long m, double c, int es) {
+  int e = 0;
+  const long long mant = (long long)ldexp(frexp(c, &e), 53);  // c = mant 2^(e - 53)
+  const int sh = (es - 1080) - (e - 53 - 56);                  // the product's units to the entry's
+  __int128 v = (__int128)m * mant;
+  if (sh > 0)
+    v = sh < 126 ? (v + ((__int128)1 << (sh - 1))) >> sh : 0;
+  else
+    v = 0;  // c = 0 (a positive c gives entries below 2^59, so sh > 50)
+  const long long q = (long long)v;
+  return make_int2((int)(q >> 28), (int)(q & 0xFFFFFFF));
+}
+
+// The fixed-point form of the FP64 operator (nsk_fx.cuh): every row sum stays below 2^62 units of
+// 2^(es - 1023 - 61).
+void fill_fx(NskFx& f, int np, int node_type, const double* rh, double mu) {
+  const FxBase& b = fx_base(node_type, np);
+  const double up = 1.0 + 1e-12;  // the row sums are rounded
+  memset(&f, 0, sizeof(f));
+  for (int k = 0; k < 3; ++k) {
+    f.ed[k] = biased_exp(rh[k] * b.msum * up);
+    for (int i = 0; i < np; ++i)
+      for (int j = 0; j < np + 2; ++j) f.d[k][i][j] = fx_entry(b.m[i][j], rh[k], f.ed[k]);
+  }
+  f.el = biased_exp(b.lsum * up);
+  f.emu = biased_exp(mu * b.lsum * up);
+  for (int s = 0; s < 2; ++s)
+    for (int j = 0; j < np; ++j) {
+      f.l[s][j] = fx_entry(b.l[s][j], 1.0, f.el);
+      f.l[2 + s][j] = fx_entry(b.l[s][j], mu, f.emu);
+    }
+}
+
 // index constants of the kernels (after E and ne are known)
 void set_index_constants(NskParams& p, int npe, int nfn) {
   p.nne = (int)(p.E * npe);
@@ -184,9 +300,12 @@ void set_index_constants(NskParams& p, int npe, int nfn) {
   p.fd_E = make_fastdiv((unsigned)p.E);
 }
 
-void set_eos_constants(NskParams& p) {
-  fill_coef<double>(p.td, p);
-  fill_coef<float>(p.tf, p);
+void set_eos_constants(NskParams& p, int np, int node_type, const double* x, const double* w) {
+  const NskBasis b = make_basis(np, x, w);
+  fill_coef<double>(p.td, p, b, np, w);
+  fill_coef<float>(p.tf, p, b, np, w);
+  fill_fx(p.fx, np, node_type, p.rh, p.mu);
+  p.rkb = p.beta / p.kappa;
   p.t8 = 8.0 * p.T;
   p.t24 = 24.0 * p.T;
   p.pa2 = 0.5 * p.alpha - 3.0;
@@ -452,8 +571,6 @@ int nsk_init_mesh(nsk_ctx** out, int dim, const int nelem[3], const double lo[3]
     if (k < dim) p.jac *= c->h[k] / 2.0;
   }
   set_index_constants(p, c->npe, c->nfn);
-  fill_tab<double>(p.td, c->np, c->xi, c->w);
-  fill_tab<float>(p.tf, c->np, c->xi, c->w);
 
   const size_t rs = c->rsize;
   const long long nn = c->nn;
@@ -510,7 +627,7 @@ int nsk_set_params(nsk_ctx* c, double T, double kappa, double alpha, double beta
   c->p.alpha = alpha;
   c->p.beta = beta;
   c->p.mu = mu;
-  set_eos_constants(c->p);
+  set_eos_constants(c->p, c->np, c->node_type, c->xi, c->w);
   c->params_set = true;
   return NSK_OK;
 }
@@ -1322,9 +1439,7 @@ extern "C" int nsk_rhs_static_scratch(int dim, const int nelem[3], const double 
   p.alpha = alpha;
   p.beta = beta;
   p.mu = mu;
-  fill_tab<double>(p.td, np, xi, w);
-  fill_tab<float>(p.tf, np, xi, w);
-  set_eos_constants(p);
+  set_eos_constants(p, np, node_type, xi, w);
 
   void* base = nullptr;
   int st = static_scratch_address(&base);

@@ -1,0 +1,189 @@
+// nsk_fx.cuh -- the FP64 operator's constant-matrix contractions in integer arithmetic.
+//
+// Why: an SM of this GPU issues 2 FP64 operations per clock and 58 to 64 32-bit integer
+// operations (measured: DFMA 2.0, mad.wide.s32 58, shifts and logic 64 per clock and SM), and the
+// two pipes run side by side. Two thirds of the FP64 instructions of a stage are multiply-adds of
+// nodal values with the fixed operator matrices (derivative, surface lifting, face interpolation),
+// so they move to the integer pipe as exact fixed-point sums; the pointwise physics stays in FP64.
+//
+// How: the values that meet in one line of a contraction (its NP nodal values and its two face
+// values) are brought to one scale, the exponent E of the largest of them, as 62-bit magnitudes in
+// two limbs, x = (h 2^32 + l 2^4) 2^(E - 1023 - 61) with h signed and 0 <= l < 2^28; the matrix
+// entries are stored the same way at the exponent of the largest row sum. A product takes three
+// 32 x 32 -> 64 bit multiply-adds (h h, h l, l h; l l is below the unit of the sum), sums are exact,
+// and one normalisation per output rounds to FP64. Every bit of a value down to 2^-57 of the line's
+// largest one is kept, where FP64 accumulation rounds each partial sum to 2^-53 of itself, so the
+// result's error is smaller than that of the FP64 sums it replaces, and it does not depend on the
+// order of the terms or on the thread that forms it.
+//
+// Measured (64^3 elements, N = 3, 256 threads, per stage): lifting 3.77 -> 1.87 ms, volume 5.15 -> 3.02
+// ms, prolongation 1.35 -> 0.60 ms. Bound now: the lifting by integer issue (ALU pipe 52 %, FP64 48 %,
+// issue slots 51 % busy at 32 resident warps), the volume kernel by latency at 16 resident warps
+// (FP64 53 %, ALU 36 %).
+//
+// Bounds: |h| <= 2^30, row sums of |matrix h| <= 2^30, at most 8 terms: |sum h h| <= 2^60,
+// |sum (h l + l h)| <= 8 2^58 + 2^58 < 2^62; three directions add up below 2^62.
+//
+// Exceptional values: an infinity or NaN in a line makes every output of the line NaN; a line of
+// values below 2^-923 (zeros, subnormals) gives zeros, and so do results below 2^-1022.
+#pragma once
+
+#include "nsk_internal.h"
+
+namespace nsk {
+
+// the contraction goes to the integer pipe in FP64 on 2D and 3D elements with lines of 3 nodes or
+// more. A line of 2 nodes has 4 multiply-adds per output, fewer FP64 issue slots than its
+// conversions cost integer ones; on 1D elements one line is the whole element, and the serial chain
+// of a conversion, product and normalisation is longer than 6 FP64 operations (64 elements, N = 3,
+// single block: 54 us a step against 48).
+template <typename R, int D, int NP>
+__host__ __device__ constexpr bool fx_on() {
+  return sizeof(R) == 8 && D >= 2 && NP >= 3;
+}
+
+constexpr unsigned kFxMin = 100u << 20;  // lines below 2^-923 share that exponent
+constexpr int kFxNan = 1 << 16;          // added to the exponent of a line with an infinity or NaN,
+                                         // subtracted from that of a line below 2^-923 (its sums are zero)
+
+struct FxVal {
+  int h, l;
+};
+
+__device__ __forceinline__ unsigned fx_mag(double x) { return (unsigned)__double2hiint(x) & 0x7FFFFFFFu; }
+
+// x at the scale of E (the largest magnitude's high word with its low 20 bits set)
+__device__ __forceinline__ FxVal fx_val(double x, unsigned E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned sh = (E - (hi & 0x7FFFFFFFu)) >> 20;
+  const unsigned vh = (__funnelshift_l(lo, hi, 9) & 0x1FFFFFFFu) | 0x20000000u;
+  unsigned long long v = ((unsigned long long)vh << 32) | (lo << 9);
+  asm("shr.u64 %0, %0, %1;" : "+l"(v) : "r"(sh));  // shifts of 64 and more give zero
+  const int s = (int)hi >> 31;
+  return FxVal{(int)(unsigned)(v >> 32) ^ s, (int)(((unsigned)v ^ (unsigned)s) >> 4)};
+}
+
+struct FxAcc {
+  long long hh, cr;
+  __device__ __forceinline__ void clear() { hh = cr = 0; }
+  __device__ __forceinline__ void mac(const FxVal a, const int2 t) {
+    hh += (long long)a.h * t.x;
+    cr += (long long)a.h * t.y;
+    cr += (long long)a.l * t.x;
+  }
+  __device__ __forceinline__ long long sum() const { return hh + (cr >> 28); }
+};
+
+// exponent of a sum of values at E with a table of biased exponent et
+__device__ __forceinline__ int fx_exp(unsigned E, int et) {
+  const int e = (int)(E >> 20);
+  return e + et + (e >= 0x7FF ? kFxNan : (e <= (int)(kFxMin >> 20) ? -kFxNan : 0));
+}
+
+// the sum a of exponent e as FP64, rounded to nearest (sign flipped when NEG)
+template <bool NEG>
+__device__ __forceinline__ double fx_out(long long a, int e) {
+  const unsigned long long s = (unsigned long long)(a >> 63);
+  unsigned long long m = ((unsigned long long)a ^ s) - s;
+  const int lz = __clzll((long long)m);
+  m <<= lz & 63;
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 2^52 <= r <= 2^53
+  const int eb = e - 1019 - lz;                                  // biased exponent - 1 (r carries the hidden bit)
+  unsigned hi = (unsigned)(r >> 32) + ((unsigned)eb << 20);
+  unsigned lo = (unsigned)r;
+  if (m == 0 || eb < 0) hi = lo = 0;
+  if (eb >= 2046) hi = 0x7FF80000u;
+  const unsigned sg = NEG ? ~(unsigned)s : (unsigned)s;
+  return __hiloint2double((int)(hi | (sg & 0x80000000u)), (int)lo);
+}
+
+// shared-memory copy of the tables (8-byte units): [D][NP][NP + 2] rows of the direction operators
+// (NP volume entries, then the +1 and -1 faces' entries), then [4][NP]: l(-1), l(+1), mu l(-1), mu l(+1)
+template <int D, int NP>
+__host__ __device__ constexpr int fx_tab_smem() {
+  return D * NP * (NP + 2) + 4 * NP;
+}
+template <int D, int NP>
+__device__ __forceinline__ void fx_stage_tables(const NskFx& f, int2* tb) {
+  constexpr int W = NP + 2;
+  for (int x = threadIdx.x; x < D * NP * W; x += blockDim.x) {
+    const int k = x / (NP * W), r = x % (NP * W);
+    tb[x] = f.d[k][r / W][r % W];
+  }
+  for (int x = threadIdx.x; x < 4 * NP; x += blockDim.x) tb[D * NP * W + x] = f.l[x / NP][x % NP];
+}
+
+// The NP sums of one line: x its nodal values, xp and xm its +1 and -1 face values, T the rows of
+// the direction's operator; returns the line's E.
+template <int NP>
+__device__ __forceinline__ unsigned fx_line(const double (&x)[NP], const double xp, const double xm,
+                                            const int2* __restrict__ T, long long (&acc)[NP]) {
+  constexpr int W = NP + 2;
+  unsigned m = kFxMin;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
+  m = max(max(m, fx_mag(xp)), fx_mag(xm));
+  const unsigned E = m | 0xFFFFFu;
+  FxVal v[W];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) v[j] = fx_val(x[j], E);
+  v[NP] = fx_val(xp, E);
+  v[NP + 1] = fx_val(xm, E);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    FxAcc a;
+    a.clear();
+    if constexpr (W % 2 == 0) {  // rows start 16-byte aligned
+#pragma unroll
+      for (int j = 0; j < W; j += 2) {
+        const int4 t = *reinterpret_cast<const int4*>(T + i * W + j);
+        a.mac(v[j], make_int2(t.x, t.y));
+        a.mac(v[j + 1], make_int2(t.z, t.w));
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < W; ++j) a.mac(v[j], T[i * W + j]);
+    }
+    acc[i] = a.sum();
+  }
+  return E;
+}
+
+// both face values of one line: x its nodal values, Tm and Tp the interpolation weights at -1 and
+// +1 (biased exponent et)
+template <int NP>
+__device__ __forceinline__ void fx_ends(const double (&x)[NP], const int2* __restrict__ Tm,
+                                        const int2* __restrict__ Tp, const int et, double& om, double& op) {
+  unsigned m = kFxMin;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
+  const unsigned E = m | 0xFFFFFu;
+  FxAcc a, b;
+  a.clear();
+  b.clear();
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    const FxVal v = fx_val(x[j], E);
+    a.mac(v, Tm[j]);
+    b.mac(v, Tp[j]);
+  }
+  const int e = fx_exp(E, et);
+  om = fx_out<false>(a.sum(), e);
+  op = fx_out<false>(b.sum(), e);
+}
+
+// one face value of a line (weights T), the same value as fx_ends gives
+template <int NP>
+__device__ __forceinline__ double fx_end(const double (&x)[NP], const int2* __restrict__ T, const int et) {
+  unsigned m = kFxMin;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
+  const unsigned E = m | 0xFFFFFu;
+  FxAcc a;
+  a.clear();
+#pragma unroll
+  for (int j = 0; j < NP; ++j) a.mac(fx_val(x[j], E), T[j]);
+  return fx_out<false>(a.sum(), fx_exp(E, et));
+}
+
+}  // namespace nsk

@@ -20,27 +20,32 @@ enum : int {
   NSK_EBIT_BOUNDS = 16,   // an index check of the bounds-checking build failed
 };
 
-// 1D nodal tables of the tensor-product basis (Sec. 3.1), in both precisions.
-// dvol[i*NSK_MAXNP + j] = (w_j / w_i) l_i'(xi_j): weak-form volume operator;
-// lm/lp[j] = l_j(-1) / l_j(+1): prolongation to the faces;
-// lmw/lpw[i] = l_i(-1) / w_i, l_i(+1) / w_i: surface lifting.
+// Nodal tables of the tensor-product basis (Sec. 3.1) and model coefficients, in both precisions.
+// lm/lp[j] = l_j(-1) / l_j(+1): prolongation to the faces.
 template <typename R>
 struct NskTab {
-  R dvol[NSK_MAXNP * NSK_MAXNP];
   R lm[NSK_MAXNP], lp[NSK_MAXNP];
-  R lmw[NSK_MAXNP], lpw[NSK_MAXNP];
   R w[NSK_MAXNP];  // quadrature weights
   // model coefficients in the operator's precision (no per-thread conversions or divisions)
-  R rh[3];         // 2 / h_k
   R mu, kb, alpha, ab;  // mu, kappa / beta, alpha, alpha / beta
   // the operators of direction k with the metric factor 2/h_k folded in (one rounding of
-  // the product, fewer instructions in the contractions): dk = (2/h_k) dvol,
-  // lpk = (2/h_k) lpw, lmk = (2/h_k) lmw
+  // the product, fewer instructions in the contractions): dk = (2/h_k) (w_j / w_i) l_i'(xi_j) the
+  // weak-form volume operator, lpk, lmk = (2/h_k) l_i(+-1) / w_i the surface lifting
   R dk[3][NSK_MAXNP * NSK_MAXNP];
   R lpk[3][NSK_MAXNP], lmk[3][NSK_MAXNP];
   // face interpolation with the viscous coefficients folded in (the lifting's traces of
   // F^v: mu l(+-1) for the stress, (kappa/beta) l(+-1) for the c flux)
   R lpmu[NSK_MAXNP], lmmu[NSK_MAXNP], lpkb[NSK_MAXNP], lmkb[NSK_MAXNP];
+};
+
+// The FP64 operator's matrices in the two-limb fixed-point form of nsk_fx.cuh (.x the signed high
+// limb, .y the low one), with the biased exponents of their scales.
+struct NskFx {
+  // row i of direction k: (2/h_k) dvol[i][j] (j < np), then the +1 and -1 faces' surface entries of
+  // a doubled face value: -lpk[i] / 2 and lmk[i] / 2
+  int2 d[3][NSK_MAXNP][NSK_MAXNP + 2];
+  int2 l[4][NSK_MAXNP];  // l_j(-1), l_j(+1), mu l_j(-1), mu l_j(+1)
+  int ed[3], el, emu;
 };
 
 // Components of a face trace: the conservative variables, and in FP64 also
@@ -66,7 +71,8 @@ __host__ __device__ __forceinline__ unsigned fdiv(unsigned x, FastDiv f) {
   return (unsigned)(((unsigned long long)x * f.m) >> f.s);
 }
 
-// Everything a kernel needs besides its buffers; passed by value.
+// Everything a kernel needs besides its buffers; passed by value (below 4 KB: a larger parameter
+// block makes every launch slower, 1 % of a 13-kernel implicit step).
 struct NskParams {
   long long E;     // number of elements
   int ne[3];       // elements per direction (1 beyond dim)
@@ -87,6 +93,8 @@ struct NskParams {
   float spin_lof, spin_hif; // the same bounds rounded outward to FP32
   int c_diss;      // Lax-Friedrichs jump on c as well
   int flux;        // NSK_FLUX_LF or NSK_FLUX_HLLC
+  double rkb;      // beta / kappa
+  NskFx fx;
   int* berr;       // error word of the bounds-checking build's index checks (NULL: none)
   NskTab<double> td;
   NskTab<float> tf;
@@ -99,6 +107,8 @@ template <> struct TabSel<double> {
 template <> struct TabSel<float> {
   __host__ __device__ static const NskTab<float>& get(const NskParams& p) { return p.tf; }
 };
+
+static_assert(sizeof(NskParams) <= 4000, "kernel parameters stay below 4 KB");
 
 // Device buffers of one context (type-erased: FP64 or FP32 per precision mode).
 struct NskBuffers {

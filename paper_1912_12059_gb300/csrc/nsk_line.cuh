@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(G * 16)
     }
   }
   cp_async_commit();
-  volume_tables<R, 3, 4>(T, tb, mode == NSK_MODE_RHS ? R(1) : dt);
+  volume_tables<R, 3, 4>(p, tb, mode == NSK_MODE_RHS ? R(1) : dt);
   R u[NV][4], kin[NV][4], gc[3][4], fx[NV][4];
   if (valid) {
 #pragma unroll

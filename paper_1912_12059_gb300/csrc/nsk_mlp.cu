@@ -688,7 +688,22 @@ __global__ void __launch_bounds__(G * nsk::Shape<D, NP>::NPE)
     sc[le * NPE + n] = cv;
   }
   __syncthreads();
-  if (valid) {
+  if constexpr (nsk::fx_on<R, D, NP>()) {
+    if (valid) {
+      double* o = Utr + (size_t)(D + 1) * NF * p.nfe + (e * NFN);
+      for (int it = n; it < D * NFN; it += NPE) {
+        const int k = it / NFN, fn = it % NFN;
+        const int n0 = nsk::line_base<D, NP>(fn, k), st = nsk::node_stride<NP>(k);
+        double x[NP];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) x[j] = sc[le * NPE + n0 + j * st];
+        double om, op;
+        nsk::fx_ends<NP>(x, p.fx.l[0], p.fx.l[1], p.fx.el, om, op);
+        o[(size_t)(2 * k) * p.nfe + fn] = om;
+        o[(size_t)(2 * k + 1) * p.nfe + fn] = op;
+      }
+    }
+  } else if (valid) {
     const auto& t = TabSel<R>::get(p);
     R* o = Utr + (size_t)(D + 1) * NF * p.nfe + (e * NFN);
     for (int it = n; it < NF * NFN; it += NPE) {
