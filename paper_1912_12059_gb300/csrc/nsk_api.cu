@@ -277,12 +277,9 @@ void fill_fx(NskFx& f, int np, int node_type, const double* rh, double mu) {
       for (int j = 0; j < np + 2; ++j) f.d[k][i][j] = fx_entry(b.m[i][j], rh[k], f.ed[k]);
   }
   f.el = biased_exp(b.lsum * up);
-  f.emu = biased_exp(mu * b.lsum * up);
   for (int s = 0; s < 2; ++s)
-    for (int j = 0; j < np; ++j) {
-      f.l[s][j] = fx_entry(b.l[s][j], 1.0, f.el);
-      f.l[2 + s][j] = fx_entry(b.l[s][j], mu, f.emu);
-    }
+    for (int j = 0; j < np; ++j) f.l[s][j] = fx_entry(b.l[s][j], 1.0, f.el);
+  f.mum = (long long)ldexp(frexp(mu, &f.mue), 63);
 }
 
 // index constants of the kernels (after E and ne are known)

@@ -97,20 +97,69 @@ __device__ __forceinline__ double fx_out(long long a, int e) {
   return __hiloint2double((int)(hi | (sg & 0x80000000u)), (int)lo);
 }
 
+// a >> n for sums at different exponents (n of 64 and more leaves the sign)
+__device__ __forceinline__ long long fx_shift(long long a, int n) {
+  asm("shr.s64 %0, %0, %1;" : "+l"(a) : "r"(n));
+  return a;
+}
+
+// Position of value i of line L in shared memory. Lines of 4 values are 32 bytes: the two 16-byte
+// halves of every other group of 4 lines change places, so that the 8 lanes of a 16-byte access to
+// consecutive lines fall on all 32 banks (4-way instead of 8-way without it for a warp's loads).
+template <int NP>
+__device__ __forceinline__ int fx_pos(int L, int i) {
+  return L * NP + (NP == 4 ? (i ^ ((L >> 1) & 2)) : i);
+}
+template <int NP>
+__device__ __forceinline__ void fx_load(const double* f, int L, double (&x)[NP]) {
+  if constexpr (NP % 2 == 0) {
+#pragma unroll
+    for (int j = 0; j < NP; j += 2) {
+      const double2 t = *reinterpret_cast<const double2*>(f + fx_pos<NP>(L, j));
+      x[j] = t.x;
+      x[j + 1] = t.y;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) x[j] = f[L * NP + j];
+  }
+}
+template <int NP>
+__device__ __forceinline__ void fx_store(double* f, int L, const long long (&x)[NP]) {
+  if constexpr (NP % 2 == 0) {
+#pragma unroll
+    for (int j = 0; j < NP; j += 2)
+      *reinterpret_cast<longlong2*>(f + fx_pos<NP>(L, j)) = make_longlong2(x[j], x[j + 1]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) f[L * NP + j] = __longlong_as_double(x[j]);
+  }
+}
+
 // shared-memory copy of the tables (8-byte units): [D][NP][NP + 2] rows of the direction operators
-// (NP volume entries, then the +1 and -1 faces' entries), then [4][NP]: l(-1), l(+1), mu l(-1), mu l(+1)
+// (NP volume entries, then the +1 and -1 faces' entries), then [2][NP] l(-1), l(+1), and for the
+// lifting the direction operators again, times mu
 template <int D, int NP>
 __host__ __device__ constexpr int fx_tab_smem() {
-  return D * NP * (NP + 2) + 4 * NP;
+  return D * NP * (NP + 2) + 2 * NP;
 }
 template <int D, int NP>
+__host__ __device__ constexpr int fx_tab_lift_smem() {
+  return fx_tab_smem<D, NP>() + D * NP * (NP + 2);
+}
+template <int D, int NP, bool LIFT>
 __device__ __forceinline__ void fx_stage_tables(const NskFx& f, int2* tb) {
   constexpr int W = NP + 2;
   for (int x = threadIdx.x; x < D * NP * W; x += blockDim.x) {
     const int k = x / (NP * W), r = x % (NP * W);
-    tb[x] = f.d[k][r / W][r % W];
+    const int2 v = f.d[k][r / W][r % W];
+    tb[x] = v;
+    if constexpr (LIFT) {  // the 58-bit entry times mu's 63-bit mantissa, back at 58 bits
+      const long long q = __mul64hi(((long long)v.x << 29) + ((long long)v.y << 1), f.mum);
+      tb[fx_tab_smem<D, NP>() + x] = make_int2((int)(q >> 28), (int)(q & 0xFFFFFFF));
+    }
   }
-  for (int x = threadIdx.x; x < 4 * NP; x += blockDim.x) tb[D * NP * W + x] = f.l[x / NP][x % NP];
+  for (int x = threadIdx.x; x < 2 * NP; x += blockDim.x) tb[D * NP * W + x] = f.l[x / NP][x % NP];
 }
 
 // The NP sums of one line: x its nodal values, xp and xm its +1 and -1 face values, T the rows of

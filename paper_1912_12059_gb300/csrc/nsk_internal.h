@@ -44,8 +44,9 @@ struct NskFx {
   // row i of direction k: (2/h_k) dvol[i][j] (j < np), then the +1 and -1 faces' surface entries of
   // a doubled face value: -lpk[i] / 2 and lmk[i] / 2
   int2 d[3][NSK_MAXNP][NSK_MAXNP + 2];
-  int2 l[4][NSK_MAXNP];  // l_j(-1), l_j(+1), mu l_j(-1), mu l_j(+1)
-  int ed[3], el, emu;
+  int2 l[2][NSK_MAXNP];  // l_j(-1), l_j(+1)
+  long long mum;         // mu = mum 2^(mue - 63), 2^62 <= mum < 2^63 (0: mu = 0)
+  int ed[3], el, mue;
 };
 
 // Components of a face trace: the conservative variables, and in FP64 also

@@ -527,7 +527,7 @@ class Batch:
         t, f, p, ms = C.c_int(), C.c_int(), C.c_int(), C.c_double()
         _check(load_library().nsk_batch_autotune(self.h, C.byref(t), C.byref(f), C.byref(p), C.byref(ms)),
                "nsk_batch_autotune")
-        return t.value, bool(f.value), p.value, ms.value
+        return t.value, f.value, p.value, ms.value
 
     def set_timeout(self, seconds):
         _check(load_library().nsk_batch_set_timeout(self.h, seconds), "nsk_batch_set_timeout")
