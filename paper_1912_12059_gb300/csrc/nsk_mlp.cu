@@ -82,17 +82,17 @@ extern "C" int nsk_gemm_bf16(const void* A, const void* B, int M, int N, int K, 
 #include <new>
 
 struct nsk_mlp {
-  int nin, nin_pad, h1, h2, nout, max_batch, max_rows, ldb;  // ldb: row stride of transposed activations
+  int nin, nin_pad, h1, h2, nout, max_batch, max_rows;
   cudaStream_t stream;
   size_t nparam, oW1, ob1, oW2, ob2, oW3, ob3;
   float *param, *grad, *m1, *m2;
   __nv_bfloat16 *W1, *W1t, *W2, *W2t, *W3, *W3t;
   // training activations (max_batch rows)
-  __nv_bfloat16 *Xt, *H1, *H1t, *H2, *H2t, *dY, *dYt, *dZ2, *dZ2t, *dZ1, *dZ1t;
-  float *Z1, *Z2, *Y;
+  __nv_bfloat16 *H1, *H2, *dY, *dZ2, *dZ1;
+  float *Z1, *Z2;
   // inference activations (max_rows rows)
   __nv_bfloat16 *IH1, *IH2;
-  double* loss;
+  double* loss;  // behind the gradients
   int* err;
   long long adam_step, launches;
   int fused_forward;  // 1 (default): inference forward in one kernel when the network fits
@@ -112,46 +112,33 @@ __global__ void k_weights_bf16(const float* __restrict__ W, int N, int K, __nv_b
   Wt[(size_t)k * N + n] = v;
 }
 
-__global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ X, int rows, int cols, int ldx,
-                                 __nv_bfloat16* __restrict__ Xt, int ldt) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)rows * cols) return;
-  const int r = (int)(i / cols), c = (int)(i % cols);
-  Xt[(size_t)c * ldt + r] = X[(size_t)r * ldx + c];
-}
-
-// mean squared error L = sum (Y - T)^2 / (B n); dY = 2 (Y - T) / (B n) in BF16 (and transposed);
-// column sums of dY are the gradient of the output bias
-__global__ void k_loss_grad(const float* __restrict__ Y, const float* __restrict__ T, int B, int n,
-                            __nv_bfloat16* __restrict__ dY, __nv_bfloat16* __restrict__ dYt, int ldt,
-                            float* __restrict__ gb3, double* __restrict__ loss) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  if (i < (long long)B * n) {
-    const int r = (int)(i / n), c = (int)(i % n);
-    const float d = Y[i] - T[i];
-    l = (double)d * d;
-    const float g = 2.0f * d / ((float)B * (float)n);
-    const __nv_bfloat16 gb = __float2bfloat16_rn(g);
-    dY[i] = gb;
-    dYt[(size_t)c * ldt + r] = gb;
-    atomicAdd(&gb3[c], g);
-  }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
-}
-
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// One Adam step of every parameter, and the BF16 copies of the weight matrices (as they lie and, for
+// the backward data products, transposed) that the next step multiplies, in one pass.
+struct AdamLayers {
+  __nv_bfloat16 *W[3], *Wt[3];
+  int off[3], N[3], K[3];  // offset and shape of the weight matrices in the parameter vector
+};
+__global__ void __launch_bounds__(256) k_adam(float* __restrict__ p, const float* __restrict__ g,
+                                              float* __restrict__ m, float* __restrict__ v, int n, float lr, float b1,
+                                              float b2, float eps, float c1, float c2, const AdamLayers L) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float gi = g[i];
   const float mi = b1 * m[i] + (1.0f - b1) * gi;
   const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
   m[i] = mi;
   v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  p[i] = w;
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    const int r = i - L.off[l];
+    if (r >= 0 && r < L.N[l] * L.K[l]) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(w);
+      L.W[l][r] = h;
+      L.Wt[l][(size_t)(r % L.K[l]) * L.N[l] + r / L.K[l]] = h;
+    }
+  }
 }
 
 unsigned nb(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -183,23 +170,21 @@ int mlp_weights_to_bf16(nsk_mlp* m) {
   return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
+size_t grad_bytes(const nsk_mlp* m) { return ((sizeof(float) * m->nparam + 7) & ~(size_t)7) + sizeof(double); }
+
 // forward + backward of one batch; gradients into m->grad, loss (sum of squares) into m->loss
 int mlp_grad(nsk_mlp* m, const __nv_bfloat16* X, const float* T, int B) {
   cudaStream_t s = m->stream;
   int* e = m->err;
-  if (cudaMemsetAsync(m->grad, 0, sizeof(float) * m->nparam, s) != cudaSuccess ||
-      cudaMemsetAsync(m->loss, 0, sizeof(double), s) != cudaSuccess)
-    return NSK_ERR_CUDA;
+  // one allocation: the gradients, then the loss
+  if (cudaMemsetAsync(m->grad, 0, grad_bytes(m), s) != cudaSuccess) return NSK_ERR_CUDA;
   int st;
-  k_transpose_bf16<<<nb((long long)B * m->nin_pad), 256, 0, s>>>(X, B, m->nin_pad, m->nin_pad, m->Xt, m->ldb);
   nsk::tc::GemmArgs a = gemm_args(X, m->nin_pad, m->W1, m->nin_pad, B, m->h1, m->nin_pad, nsk::tc::EPI_GELU, e);
   a.bias = m->param + m->ob1;
   a.out = m->Z1;
   a.ldo = m->h1;
   a.hout = m->H1;
   a.ldh = m->h1;
-  a.hout_t = m->H1t;
-  a.ldt = m->ldb;
   if ((st = nsk::tc::launch_gemm(a, s))) return st;
   a = gemm_args(m->H1, m->h1, m->W2, m->h1, B, m->h2, m->h1, nsk::tc::EPI_GELU, e);
   a.bias = m->param + m->ob2;
@@ -207,24 +192,25 @@ int mlp_grad(nsk_mlp* m, const __nv_bfloat16* X, const float* T, int B) {
   a.ldo = m->h2;
   a.hout = m->H2;
   a.ldh = m->h2;
-  a.hout_t = m->H2t;
-  a.ldt = m->ldb;
   if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  a = gemm_args(m->H2, m->h2, m->W3, m->h2, B, m->nout, m->h2, nsk::tc::EPI_STORE, e);
+  // mean squared error L = sum (Y - T)^2 / (B n); dY = 2 (Y - T) / (B n) in BF16; column sums of dY are
+  // the gradient of the output bias
+  a = gemm_args(m->H2, m->h2, m->W3, m->h2, B, m->nout, m->h2, nsk::tc::EPI_LOSS, e);
   a.bias = m->param + m->ob3;
-  a.out = m->Y;
-  a.ldo = m->nout;
+  a.target = T;
+  a.hout = m->dY;
+  a.ldh = m->nout;
+  a.bias_grad = m->grad + m->ob3;
+  a.loss = m->loss;
+  a.g_num = 2.0f;
+  a.g_den = (float)B * (float)m->nout;
   if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  k_loss_grad<<<nb((long long)B * m->nout), 256, 0, s>>>(m->Y, T, B, m->nout, m->dY, m->dYt, m->ldb,
-                                                          m->grad + m->ob3, m->loss);
   // dZ2 = (dY W3) * GELU'(Z2)
   a = gemm_args(m->dY, m->nout, m->W3t, m->nout, B, m->h2, m->nout, nsk::tc::EPI_DGELU, e);
   a.zin = m->Z2;
   a.ldz = m->h2;
   a.hout = m->dZ2;
   a.ldh = m->h2;
-  a.hout_t = m->dZ2t;
-  a.ldt = m->ldb;
   a.bias_grad = m->grad + m->ob2;
   if ((st = nsk::tc::launch_gemm(a, s))) return st;
   // dZ1 = (dZ2 W2) * GELU'(Z1)
@@ -233,28 +219,17 @@ int mlp_grad(nsk_mlp* m, const __nv_bfloat16* X, const float* T, int B) {
   a.ldz = m->h1;
   a.hout = m->dZ1;
   a.ldh = m->h1;
-  a.hout_t = m->dZ1t;
-  a.ldt = m->ldb;
   a.bias_grad = m->grad + m->ob1;
   if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  // weight gradients: reduction over the batch (split-K partial sums)
-  const int ks = 256;
-  a = gemm_args(m->dYt, m->ldb, m->H2t, m->ldb, m->nout, m->h2, B, nsk::tc::EPI_ATOMIC, e);
-  a.out = m->grad + m->oW3;
-  a.ldo = m->h2;
-  a.k_split = ks;
-  if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  a = gemm_args(m->dZ2t, m->ldb, m->H1t, m->ldb, m->h2, m->h1, B, nsk::tc::EPI_ATOMIC, e);
-  a.out = m->grad + m->oW2;
-  a.ldo = m->h1;
-  a.k_split = ks;
-  if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  a = gemm_args(m->dZ1t, m->ldb, m->Xt, m->ldb, m->h1, m->nin_pad, B, nsk::tc::EPI_ATOMIC, e);
-  a.out = m->grad + m->oW1;
-  a.ldo = m->nin_pad;
-  a.k_split = ks;
-  if ((st = nsk::tc::launch_gemm(a, s))) return st;
-  m->launches += 10;
+  // weight gradients: reductions over the batch
+  nsk::tc::WgradArgs w;
+  w.job[0] = {m->dZ1, X, m->grad + m->oW1, m->h1, m->nin_pad, m->h1, m->nin_pad};
+  w.job[1] = {m->dZ2, m->H1, m->grad + m->oW2, m->h2, m->h1, m->h2, m->h1};
+  w.job[2] = {m->dY, m->H2, m->grad + m->oW3, m->nout, m->h2, m->nout, m->h2};
+  w.batch = B;
+  w.err = e;
+  if ((st = nsk::tc::launch_wgrad(w, s))) return st;
+  m->launches += 6;
   return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
@@ -321,9 +296,8 @@ int mlp_check(nsk_mlp* m, double* loss_out, int B) {
 
 void mlp_free(nsk_mlp* m) {
   if (!m) return;
-  void* ptrs[] = {m->param, m->grad, m->m1, m->m2, m->W1, m->W1t, m->W2, m->W2t, m->W3, m->W3t, m->Xt, m->H1,
-                  m->H1t, m->H2, m->H2t, m->dY, m->dYt, m->dZ2, m->dZ2t, m->dZ1, m->dZ1t, m->Z1, m->Z2, m->Y,
-                  m->IH1, m->IH2, m->loss, m->err};
+  void* ptrs[] = {m->param, m->grad, m->m1, m->m2, m->W1, m->W1t, m->W2, m->W2t, m->W3, m->W3t, m->H1,
+                  m->H2, m->dY, m->dZ2, m->dZ1, m->Z1, m->Z2, m->IH1, m->IH2, m->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete m;
@@ -348,7 +322,6 @@ int nsk_mlp_create(nsk_mlp** out, int n_in, int h1, int h2, int n_out, int max_b
   m->nout = n_out;
   m->max_batch = max_batch;
   m->max_rows = max_rows;
-  m->ldb = max_batch;
   m->stream = (cudaStream_t)stream;
   m->oW1 = 0;
   m->ob1 = m->oW1 + (size_t)h1 * m->nin_pad;
@@ -362,20 +335,17 @@ int nsk_mlp_create(nsk_mlp** out, int n_in, int h1, int h2, int n_out, int max_b
     void** p;
     size_t bytes;
   } al[] = {
-      {(void**)&m->param, f4 * m->nparam}, {(void**)&m->grad, f4 * m->nparam},
+      {(void**)&m->param, f4 * m->nparam}, {(void**)&m->grad, grad_bytes(m)},
       {(void**)&m->m1, f4 * m->nparam},    {(void**)&m->m2, f4 * m->nparam},
       {(void**)&m->W1, bf * h1 * m->nin_pad}, {(void**)&m->W1t, bf * h1 * m->nin_pad},
       {(void**)&m->W2, bf * h2 * h1},      {(void**)&m->W2t, bf * h2 * h1},
       {(void**)&m->W3, bf * n_out * h2},   {(void**)&m->W3t, bf * n_out * h2},
-      {(void**)&m->Xt, bf * m->nin_pad * B}, {(void**)&m->H1, bf * B * h1},
-      {(void**)&m->H1t, bf * B * h1},      {(void**)&m->H2, bf * B * h2},
-      {(void**)&m->H2t, bf * B * h2},      {(void**)&m->dY, bf * B * n_out},
-      {(void**)&m->dYt, bf * B * n_out},   {(void**)&m->dZ2, bf * B * h2},
-      {(void**)&m->dZ2t, bf * B * h2},     {(void**)&m->dZ1, bf * B * h1},
-      {(void**)&m->dZ1t, bf * B * h1},     {(void**)&m->Z1, f4 * B * h1},
-      {(void**)&m->Z2, f4 * B * h2},       {(void**)&m->Y, f4 * B * n_out},
+      {(void**)&m->H1, bf * B * h1},       {(void**)&m->H2, bf * B * h2},
+      {(void**)&m->dY, bf * B * n_out},    {(void**)&m->dZ2, bf * B * h2},
+      {(void**)&m->dZ1, bf * B * h1},      {(void**)&m->Z1, f4 * B * h1},
+      {(void**)&m->Z2, f4 * B * h2},
       {(void**)&m->IH1, bf * R * h1},      {(void**)&m->IH2, bf * R * h2},
-      {(void**)&m->loss, sizeof(double)},  {(void**)&m->err, sizeof(int)},
+      {(void**)&m->err, sizeof(int)},
   };
   for (auto& a : al)
     if (cudaMalloc(a.p, a.bytes) != cudaSuccess) {
@@ -383,6 +353,7 @@ int nsk_mlp_create(nsk_mlp** out, int n_in, int h1, int h2, int n_out, int max_b
       mlp_free(m);
       return NSK_ERR_NOMEM;
     }
+  m->loss = (double*)((char*)m->grad + grad_bytes(m) - sizeof(double));
   if (cudaMemset(m->param, 0, f4 * m->nparam) != cudaSuccess || cudaMemset(m->m1, 0, f4 * m->nparam) != cudaSuccess ||
       cudaMemset(m->m2, 0, f4 * m->nparam) != cudaSuccess || cudaMemset(m->err, 0, sizeof(int)) != cudaSuccess) {
     mlp_free(m);
@@ -445,10 +416,12 @@ int nsk_mlp_train_step(nsk_mlp* m, const void* X, const float* T, int batch, dou
   m->adam_step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.0f - powf(b1, (float)m->adam_step), c2 = 1.0f - powf(b2, (float)m->adam_step);
-  k_adam<<<nb((long long)m->nparam), 256, 0, m->stream>>>(m->param, m->grad, m->m1, m->m2, (long long)m->nparam,
-                                                          (float)lr, b1, b2, 1e-8f, c1, c2);
+  AdamLayers L = {{m->W1, m->W2, m->W3}, {m->W1t, m->W2t, m->W3t}, {(int)m->oW1, (int)m->oW2, (int)m->oW3},
+                  {m->h1, m->h2, m->nout}, {m->nin_pad, m->h1, m->h2}};
+  k_adam<<<nb((long long)m->nparam), 256, 0, m->stream>>>(m->param, m->grad, m->m1, m->m2, (int)m->nparam, (float)lr,
+                                                          b1, b2, 1e-8f, c1, c2, L);
   m->launches += 1;
-  if ((st = mlp_weights_to_bf16(m))) return st;
+  if (cudaGetLastError() != cudaSuccess) return NSK_ERR_CUDA;
   return loss ? mlp_check(m, loss, batch) : NSK_OK;
 }
 

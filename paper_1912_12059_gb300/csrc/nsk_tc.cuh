@@ -43,6 +43,8 @@ enum Epilogue : int {
   EPI_ATOMIC = 1,  // atomicAdd(out, C): split-K partial sums
   EPI_GELU = 2,    // z = C + bias: z -> zout (FP32, optional), GELU(z) -> hout (BF16), optional transposed copy
   EPI_DGELU = 3,   // dz = C * GELU'(zin): dz -> hout (BF16) and transposed copy, column sums -> bias_grad
+  EPI_LOSS = 4,    // d = C + bias - target: g = gscale_num d / gscale_den -> hout (BF16), column sums of g ->
+                   // bias_grad, sum of d^2 -> loss (not in the public GEMM call)
 };
 
 struct GemmArgs {
@@ -60,7 +62,10 @@ struct GemmArgs {
   int ldt;
   const float* zin;        // FP32 [M][ldz] pre-activation (DGELU)
   int ldz;
-  float* bias_grad;        // [N] column sums (DGELU, optional)
+  float* bias_grad;        // [N] column sums (DGELU, optional; LOSS)
+  const float* target;     // FP32 [M][N] (LOSS)
+  double* loss;            // sum of squares (LOSS)
+  float g_num, g_den;      // the loss gradient's factors (LOSS)
   int* err;                // error word (NSK_EBIT_TIMEOUT on an expired wait)
 };
 
@@ -358,24 +363,25 @@ __host__ __device__ constexpr int rb_b_bytes(int N, int K) { return ((N * K * 2)
 constexpr int kStage = 32 * 33;  // floats of one warp's 32 x 32 staging block (padded rows)
 
 // write the 32 x 32 block held transposed in `st` (st[r * 33 + c], row r = lane of the producer)
-// to rows row0.. of a row-major matrix with 16-byte vector stores (rows beyond rows_valid skipped)
+// to rows row0.. of a row-major matrix with 16-byte vector stores (rows beyond rows_valid and
+// columns beyond ncol, a multiple of 16, skipped)
 __device__ __forceinline__ void store_block_f32(const float* st, float* out, size_t ld, int row0, int col0,
-                                                int rows_valid, int lane) {
+                                                int rows_valid, int ncol, int lane) {
 #pragma unroll
   for (int it = 0; it < 8; ++it) {
     const int r = it * 4 + (lane >> 3), c = (lane & 7) * 4;
-    if (r < rows_valid) {
+    if (r < rows_valid && c < ncol) {
       const float4 v = make_float4(st[r * 33 + c], st[r * 33 + c + 1], st[r * 33 + c + 2], st[r * 33 + c + 3]);
       *reinterpret_cast<float4*>(out + (size_t)(row0 + r) * ld + col0 + c) = v;
     }
   }
 }
 __device__ __forceinline__ void store_block_bf16(const float* st, __nv_bfloat16* out, size_t ld, int row0, int col0,
-                                                 int rows_valid, int lane) {
+                                                 int rows_valid, int ncol, int lane) {
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const int r = it * 8 + (lane >> 2), c = (lane & 3) * 8;
-    if (r < rows_valid) {
+    if (r < rows_valid && c < ncol) {
       __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) h[j] = __float2bfloat16_rn(st[r * 33 + c + j]);
@@ -384,21 +390,24 @@ __device__ __forceinline__ void store_block_bf16(const float* st, __nv_bfloat16*
   }
 }
 
-// epilogue of the resident-B kernel for 32 columns [c0, c0 + 32) of the warp's 32 rows
-// (row0 = first row, lane = row offset); outputs go through the warp's staging block
+// epilogue of the resident-B kernel for ncol (a multiple of 16, at most 32) columns [c0, c0 + ncol)
+// of the warp's 32 rows (row0 = first row, lane = row offset); outputs go through the warp's staging
+// block
 __device__ __forceinline__ void epilogue_chunk_rb(const GemmArgs& a, const int row0, const int lane, const int c0,
-                                                  const uint32_t* v, float* st) {
+                                                  const int ncol, const uint32_t* v, float* st) {
   const int m = row0 + lane;
   const int rows_valid = a.M - row0;
   const bool rv = lane < rows_valid;
+  const bool biased = (a.epi < EPI_DGELU || a.epi == EPI_LOSS) && a.bias;
+  const float bl = biased && lane < ncol ? a.bias[c0 + lane] : 0.f;  // one column's bias per lane, broadcast below
   float x[32];
 #pragma unroll
-  for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(v[j]) + ((a.epi != EPI_DGELU && a.bias) ? a.bias[c0 + j] : 0.f);
+  for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl, j);
   if (a.epi == EPI_STORE || (a.epi == EPI_GELU && a.out)) {
 #pragma unroll
     for (int j = 0; j < 32; ++j) st[lane * 33 + j] = x[j];
     __syncwarp();
-    store_block_f32(st, a.out, a.ldo, row0, c0, rows_valid, lane);
+    store_block_f32(st, a.out, a.ldo, row0, c0, rows_valid, ncol, lane);
     __syncwarp();
     if (a.epi == EPI_STORE) return;
   }
@@ -406,7 +415,7 @@ __device__ __forceinline__ void epilogue_chunk_rb(const GemmArgs& a, const int r
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
       const int r = it * 4 + (lane >> 3), c = (lane & 7) * 4;
-      if (r < rows_valid) {
+      if (r < rows_valid && c < ncol) {
         const float4 z = *reinterpret_cast<const float4*>(a.zin + (size_t)(row0 + r) * a.ldz + c0 + c);
         st[r * 33 + c] = z.x;
         st[r * 33 + c + 1] = z.y;
@@ -416,34 +425,50 @@ __device__ __forceinline__ void epilogue_chunk_rb(const GemmArgs& a, const int r
     }
     __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) x[j] = rv ? x[j] * gelu_grad(st[lane * 33 + j]) : 0.f;
+    for (int j = 0; j < 32; ++j) x[j] = rv && j < ncol ? x[j] * gelu_grad(st[lane * 33 + j]) : 0.f;
+    __syncwarp();
+  } else if (a.epi == EPI_LOSS) {  // the targets of the block (a row's columns together), then the loss
+    for (int r = 0; r < 32; ++r)
+      if (r < rows_valid && lane < ncol) st[r * 33 + lane] = a.target[(size_t)(row0 + r) * a.N + c0 + lane];
+    __syncwarp();
+    double sq = 0.0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const float d = rv && j < ncol ? x[j] - st[lane * 33 + j] : 0.f;
+      sq += (double)d * d;
+      x[j] = a.g_num * d / a.g_den;
+    }
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) atomicAdd(a.loss, sq);
     __syncwarp();
   } else {
 #pragma unroll
     for (int j = 0; j < 32; ++j) x[j] = gelu(x[j]);
   }
-  if (a.epi == EPI_DGELU && a.bias_grad) {  // column sums of the FP32 values
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      float sum = x[j];
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0) atomicAdd(&a.bias_grad[c0 + j], sum);
-    }
-  }
 #pragma unroll
   for (int j = 0; j < 32; ++j) st[lane * 33 + j] = x[j];
   __syncwarp();
-  store_block_bf16(st, a.hout, a.ldh, row0, c0, rows_valid, lane);
+  store_block_bf16(st, a.hout, a.ldh, row0, c0, rows_valid, ncol, lane);
+  if (a.epi >= EPI_DGELU && a.bias_grad && lane < ncol) {  // column sums of the FP32 values, a column per lane
+    float sum = 0.f;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) sum += st[r * 33 + lane];
+    atomicAdd(&a.bias_grad[c0 + lane], sum);
+  }
   __syncwarp();
   if (a.hout_t && rv) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) a.hout_t[(size_t)(c0 + j) * a.ldt + m] = __float2bfloat16_rn(x[j]);
+    for (int j = 0; j < 32; ++j)
+      if (j < ncol) a.hout_t[(size_t)(c0 + j) * a.ldt + m] = __float2bfloat16_rn(x[j]);
   }
 }
 
+// gridDim.y > 1: the CTAs of row y hold the 64 columns (rows of B) from 64 y on (the last row's may
+// be 16 to 48), so that a batch of few row tiles still fills the SMs; a column's sum does not depend
+// on the split. a.N then is the whole matrix's.
 __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  const int K = a.K, N = a.N;
+  const int K = a.K, n0 = blockIdx.y * 64, N = gridDim.y > 1 ? min(64, a.N - n0) : a.N;
   unsigned char* sB = smem;
   unsigned char* sA = smem + rb_b_bytes(N, K);
   float* stage = reinterpret_cast<float*>(sA + kBM * K * 2) + (threadIdx.x >> 5) * kStage;
@@ -470,7 +495,7 @@ __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) 
   const uint32_t sBa = smem_u32(sB), sAa = smem_u32(sA);
   for (int idx = threadIdx.x; idx < N * kc; idx += kRbThreads) {
     const int r = idx / kc, j = idx % kc;
-    cp_async16(sBa + core_off_k(r, j * 8, K), a.B + (size_t)r * a.ldb + j * 8, 16);
+    cp_async16(sBa + core_off_k(r, j * 8, K), a.B + (size_t)(n0 + r) * a.ldb + j * 8, 16);
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -520,10 +545,11 @@ __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) 
     if (prev_tile >= 0) {  // epilogue of the previous tile overlaps the MMAs just issued
       const int row0 = prev_tile * kBM + q * 32;
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(((i - 1) & 1) * 256);
-      for (int c0 = half * (N / 2); c0 < (half + 1) * (N / 2); c0 += 32) {
+      const int nh = N <= 64 ? 32 : N / 2;  // columns of each half of the warps
+      for (int c0 = half * nh; c0 < min(N, (half + 1) * nh); c0 += 32) {
         uint32_t v[32];
         tmem_ld32(base + (uint32_t)c0, v);
-        epilogue_chunk_rb(a, row0, lane, c0, v, stage);
+        epilogue_chunk_rb(a, row0, lane, n0 + c0, min(32, N - c0), v, stage);
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
     }
@@ -533,6 +559,134 @@ __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) 
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// ---------------------------------------------------------------------------
+// Weight gradients of up to three layers in one launch: G_l += A_l^T B_l, A_l [batch][lda] the
+// output-side gradients (dz), B_l [batch][ldb] the layer's inputs, both row-major BF16, G_l FP32
+// [M][N]. Blocks: x = (layer, 128-row tile of its G), y = a slice of the batch (the reduction). Both
+// operands are read as they lie: batch is the K of the MMA and their columns are contiguous, i.e.
+// they are MN-major operands (instruction descriptor bits 15 and 16), so no transposed copies are
+// written or read. Shared-memory layout per operand, 128-byte core matrices of 8 batch rows x 8
+// columns, [batch / 8][columns / 8]: LBO = distance of 8 batch rows, SBO = 128 between column groups.
+// The partial sums are added to G with 16-byte reductions.
+// Bound by the operands' copies from L2 and the reductions; 96 KB of operands keep two blocks on an
+// SM (2 x 256 TMEM columns).
+// ---------------------------------------------------------------------------
+struct WgradJob {
+  const __nv_bfloat16 *A, *B;
+  float* G;
+  int M, N, lda, ldb;
+};
+struct WgradArgs {
+  WgradJob job[3];
+  int tile0[4];  // first x block of each layer, then the total
+  int batch, ks; // rows of one slice (a multiple of 16, at most kWgK)
+  int* err;
+};
+constexpr int kWgK = 128;
+constexpr int kWgThreads = 256;
+constexpr int kWgSmem = kWgK * (kBM + kMaxN) * 2;
+
+// rows [b0, b0 + nb) and columns [c0, c0 + ncol) of a row-major BF16 matrix into the layout above (column
+// groups ng = ncols / 8 wide); rows beyond nv and columns beyond cv are zero
+__device__ __forceinline__ void wg_stage(uint32_t s, const __nv_bfloat16* g, int ld, int b0, int nb, int nv, int c0,
+                                         int ng, int cv) {
+  for (int i = threadIdx.x; i < nb * ng; i += kWgThreads) {
+    const int r = i / ng, q = i % ng;
+    const bool v = r < nv && c0 + q * 8 < cv;
+    cp_async16(s + (uint32_t)(((r >> 3) * ng + q) * 128 + (r & 7) * 16),
+               v ? (const void*)(g + (size_t)(b0 + r) * ld + c0 + q * 8) : (const void*)g, v ? 16 : 0);
+  }
+}
+__device__ __forceinline__ void red_add_v4(float* p, float4 v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const WgradArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long mbar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int aborted;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int l = 0;
+  while ((int)blockIdx.x >= a.tile0[l + 1]) ++l;
+  const WgradJob& j = a.job[l];
+  const int m0 = ((int)blockIdx.x - a.tile0[l]) * kBM, b0 = blockIdx.y * a.ks;
+  const int nv = min(a.ks, a.batch - b0);
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(kMaxN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (threadIdx.x == 0) {
+    aborted = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  const uint32_t sA = smem_u32(smem), sB = sA + kWgK * kBM * 2;
+  wg_stage(sA, j.A, j.lda, b0, a.ks, nv, m0, kBM / 8, j.M);
+  wg_stage(sB, j.B, j.ldb, b0, a.ks, nv, 0, j.N / 8, j.N);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = tmem_slot;
+  if (threadIdx.x == 0) {
+    const uint32_t idesc = idesc_bf16(kBM, j.N) | (1u << 15) | (1u << 16);
+    const uint32_t la = kBM / 8 * 128, lb = (uint32_t)j.N / 8 * 128;
+    for (int s = 0; s < a.ks / 16; ++s) {  // a K step of 16 spans two core matrices along the batch
+      const uint64_t ad = sdesc(sA + s * 2 * la, la, 128), bd = sdesc(sB + s * 2 * lb, lb, 128);
+      const uint32_t acc = s > 0 ? 1u : 0u;
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+          "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+    }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+        smem_u32(&mbar)));
+  }
+  const bool ok = mbar_wait(smem_u32(&mbar), 0, a.err);
+  if (!ok) aborted = 1;
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  __syncthreads();  // the operands' shared memory is free: it stages the blocks below
+  if (!aborted) {
+    float* st = reinterpret_cast<float*>(smem) + warp * kStage;
+    const int q = warp & 3, half = warp >> 2, row0 = m0 + q * 32;
+    for (int c0 = half * 32; c0 < j.N; c0 += 64) {
+      uint32_t v[32];
+      tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) st[lane * 33 + i] = __uint_as_float(v[i]);
+      __syncwarp();
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        const int r = it * 4 + (lane >> 3), c = (lane & 7) * 4;
+        if (row0 + r < j.M && c0 + c < j.N)
+          red_add_v4(j.G + (size_t)(row0 + r) * j.N + c0 + c,
+                     make_float4(st[r * 33 + c], st[r * 33 + c + 1], st[r * 33 + c + 2], st[r * 33 + c + 3]));
+      }
+      __syncwarp();
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMaxN));
+}
+
+// slices of the batch: 128 rows (about one block per SM and layer tile at 4096 rows)
+inline int launch_wgrad(WgradArgs& a, cudaStream_t s) {
+  static const bool ok =
+      cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem) == cudaSuccess;
+  if (!ok) return NSK_ERR_CUDA;
+  a.tile0[0] = 0;
+  for (int l = 0; l < 3; ++l) a.tile0[l + 1] = a.tile0[l] + (a.job[l].M + kBM - 1) / kBM;
+  a.ks = a.batch < kWgK ? a.batch : kWgK;
+  k_wgrad<<<dim3((unsigned)a.tile0[3], (unsigned)((a.batch + a.ks - 1) / a.ks)), kWgThreads, kWgSmem, s>>>(a);
+  return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------
@@ -1298,14 +1452,22 @@ inline int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   }
   // resident-B kernel: 16-byte aligned rows of every output it writes with vector stores
   auto a16 = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
+  const int ntiles = (a.M + kBM - 1) / kBM;
   const bool aligned = (a.epi == EPI_STORE ? (a.ldo % 4) == 0 && a16(a.out) : (a.ldh % 8) == 0 && a16(a.hout)) &&
                        (!(a.epi == EPI_GELU && a.out) || ((a.ldo % 4) == 0 && a16(a.out))) &&
                        (a.epi != EPI_DGELU || ((a.ldz % 4) == 0 && a16(a.zin)));
-  const bool resident = a.epi != EPI_ATOMIC && a.k_split >= a.K && a.K <= 256 && (a.N % 64) == 0 && aligned;
-  if (resident) {
+  const bool resident = a.epi != EPI_ATOMIC && a.k_split >= a.K && a.K <= 256 && aligned;
+  // few row tiles: 64-column slices fill the SMs (4096 rows of a 256 x 256 layer: 128 blocks instead of
+  // 32, each with a quarter of the epilogue); many: one block per SM holds the whole B
+  const int ny = (a.N + 63) / 64;
+  if (resident && (ntiles * ny <= sms || a.N % 64)) {
+    int smem = rb_b_bytes(64, a.K) + kBM * a.K * 2 + kRbStageBytes;
+    smem = smem < kRbSmemMin ? kRbSmemMin : smem;
+    const int gx = (int)persistent_grid(ntiles, sms / ny > 0 ? sms / ny : 1);
+    k_gemm_tc_rb<<<dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s>>>(a);
+  } else if (resident) {
     int smem = rb_b_bytes(a.N, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
-    const int ntiles = (a.M + kBM - 1) / kBM;
     if (smem > kRbSmemMax) return NSK_ERR_ARG;
     k_gemm_tc_rb<<<persistent_grid(ntiles, sms), kRbThreads, smem, s>>>(a);
   } else {
