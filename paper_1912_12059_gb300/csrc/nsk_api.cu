@@ -188,16 +188,17 @@ void fill_coef(NskTab<R>& t, const NskParams& p, const NskBasis& td, int n, cons
 }
 
 // The reference operator in extended precision as integers of 2^-56 (exact to 58 bits of a row's
-// sum, which the fixed-point tables of nsk_fx.cuh keep): row i the np volume entries
-// (w_j / w_i) l_i'(x_j), then -l_i(+1) / (2 w_i) and l_i(-1) / (2 w_i); l: l_j(-1), l_j(+1); and
-// the largest row sums. Formed once per node set and order.
+// sum, which the fixed-point tables of nsk_fx.cuh keep), in the order of NskFx: of the rows
+// l_i(-1) / (2 w_i), the np volume entries (w_j / w_i) l_i'(x_j), -l_i(+1) / (2 w_i), and of l_j(+1); and the
+// largest row sums. Formed once per node set and order.
 struct FxBase {
-  long long m[NSK_MAXNP][NSK_MAXNP + 2], l[2][NSK_MAXNP];
+  long long m[4 * NSK_MAXNP], l[NSK_MAXNP];
+  int nm;
   double msum, lsum;
 };
 void make_fx_base(FxBase& b, int node_type, int np) {
   typedef long double T;
-  T x[NSK_MAXNP], w[NSK_MAXNP], lam[NSK_MAXNP], M[NSK_MAXNP][NSK_MAXNP + 2], l[2][NSK_MAXNP];
+  T x[NSK_MAXNP], w[NSK_MAXNP], lam[NSK_MAXNP], M[NSK_MAXNP][NSK_MAXNP], l[2][NSK_MAXNP];
   if (node_type == NSK_NODES_GAUSS)
     gauss_legendre(np, x, w);
   else
@@ -214,26 +215,28 @@ void make_fx_base(FxBase& b, int node_type, int np) {
     M[i][i] = diag;
     l[0][i] = lagrange_at(np, x, lam, i, (T)-1.0);
     l[1][i] = lagrange_at(np, x, lam, i, (T)1.0);
-    M[i][np] = (T)-0.5 * l[1][i] / w[i];
-    M[i][np + 1] = (T)0.5 * l[0][i] / w[i];
   }
+  const int W = np + 2;
   b.msum = b.lsum = 0.0;
-  for (int i = 0; i < np; ++i) {
+  b.nm = 0;
+  for (int i = 0; i < np - np / 2; ++i) {
+    T row[NSK_MAXNP + 2];
+    row[0] = (T)0.5 * l[0][i] / w[i];
+    for (int j = 0; j < np; ++j) row[1 + j] = M[i][j];
+    row[W - 1] = (T)-0.5 * l[1][i] / w[i];
     double r = 0.0;
-    for (int j = 0; j < np + 2; ++j) {
-      b.m[i][j] = llrintl(ldexpl(M[i][j], 56));
-      r += std::fabs((double)M[i][j]);
-    }
+    for (int j = 0; j < W; ++j) r += std::fabs((double)row[j]);
     b.msum = std::fmax(b.msum, r);
+    for (int j = 0; j < W / 2; ++j) b.m[b.nm++] = llrintl(ldexpl((row[j] - row[W - 1 - j]) / 2, 56));
+    if (i == np / 2) break;  // the middle row of an odd np: differences only
+    for (int j = 0; j < W / 2; ++j) b.m[b.nm++] = llrintl(ldexpl((row[j] + row[W - 1 - j]) / 2, 56));
+    if (W % 2) b.m[b.nm++] = llrintl(ldexpl(row[W / 2], 56));
   }
-  for (int s = 0; s < 2; ++s) {
-    double r = 0.0;
-    for (int j = 0; j < np; ++j) {
-      b.l[s][j] = llrintl(ldexpl(l[s][j], 56));
-      r += std::fabs((double)l[s][j]);
-    }
-    b.lsum = std::fmax(b.lsum, r);
-  }
+  for (int j = 0; j < np; ++j) b.lsum += std::fabs((double)l[1][j]);
+  int n = 0;
+  for (int j = 0; j < np / 2; ++j) b.l[n++] = llrintl(ldexpl((l[1][j] + l[1][np - 1 - j]) / 2, 56));
+  if (np % 2) b.l[n++] = llrintl(ldexpl(l[1][np / 2], 56));
+  for (int j = 0; j < np / 2; ++j) b.l[n++] = llrintl(ldexpl((l[1][j] - l[1][np - 1 - j]) / 2, 56));
 }
 const FxBase& fx_base(int node_type, int np) {
   static FxBase base[2][NSK_MAXNP + 1];
@@ -273,12 +276,10 @@ void fill_fx(NskFx& f, int np, int node_type, const double* rh, double mu) {
   memset(&f, 0, sizeof(f));
   for (int k = 0; k < 3; ++k) {
     f.ed[k] = biased_exp(rh[k] * b.msum * up);
-    for (int i = 0; i < np; ++i)
-      for (int j = 0; j < np + 2; ++j) f.d[k][i][j] = fx_entry(b.m[i][j], rh[k], f.ed[k]);
+    for (int j = 0; j < b.nm; ++j) f.d[k][j] = fx_entry(b.m[j], rh[k], f.ed[k]);
   }
   f.el = biased_exp(b.lsum * up);
-  for (int s = 0; s < 2; ++s)
-    for (int j = 0; j < np; ++j) f.l[s][j] = fx_entry(b.l[s][j], 1.0, f.el);
+  for (int j = 0; j < np; ++j) f.l[j] = fx_entry(b.l[j], 1.0, f.el);
   f.mum = (long long)ldexp(frexp(mu, &f.mue), 63);
 }
 

@@ -11,7 +11,9 @@
 // two limbs, x = (h 2^32 + l 2^4) 2^(E - 1023 - 61) with h signed and 0 <= l < 2^28; the matrix
 // entries are stored the same way at the exponent of the largest row sum. A product takes three
 // 32 x 32 -> 64 bit multiply-adds (h h, h l, l h; l l is below the unit of the sum), sums are exact,
-// and one normalisation per output rounds to FP64. Every bit of a value down to 2^-57 of the line's
+// and one normalisation per output rounds to FP64. Nodes and weights are symmetric about the centre of
+// the line, so the rows i and NP - 1 - i share their products: one of the sums, one of the differences of
+// the line's value pairs (exact), half the multiply-adds of the plain rows. Every bit of a value down to 2^-57 of the line's
 // largest one is kept, where FP64 accumulation rounds each partial sum to 2^-53 of itself, so the
 // result's error is smaller than that of the FP64 sums it replaces, and it does not depend on the
 // order of the terms or on the thread that forms it.
@@ -21,8 +23,10 @@
 // issue slots 51 % busy at 32 resident warps), the volume kernel by latency at 16 resident warps
 // (FP64 53 %, ALU 36 %).
 //
-// Bounds: |h| <= 2^30, row sums of |matrix h| <= 2^30, at most 8 terms: |sum h h| <= 2^60,
-// |sum (h l + l h)| <= 8 2^58 + 2^58 < 2^62; three directions add up below 2^62.
+// Bounds: |h| <= 2^30, pair sums and differences in [-2^31, 2^31 - 1] and their low limbs below 2^29 in
+// magnitude, row sums of |matrix h| <= 2^30, at most 4 terms a product sum: |sum h h| <= 2^61,
+// |sum (h l + l h)| <= 4 2^59 + 2^59 < 2^62; a row's result is below 2^60 and three directions add up below
+// 2^62.
 //
 // Exceptional values: an infinity or NaN in a line makes every output of the line NaN; a line of
 // values below 2^-923 (zeros, subnormals) gives zeros, and so do results below 2^-1022.
@@ -136,73 +140,102 @@ __device__ __forceinline__ void fx_store(double* f, int L, const long long (&x)[
   }
 }
 
-// shared-memory copy of the tables (8-byte units): [D][NP][NP + 2] rows of the direction operators
-// (NP volume entries, then the +1 and -1 faces' entries), then [2][NP] l(-1), l(+1), and for the
-// lifting the direction operators again, times mu
+// entries of one direction's operator (NskFx)
+template <int NP>
+__host__ __device__ constexpr int fx_entries() {
+  return (NP / 2) * (NP + 2) + (NP % 2) * ((NP + 2) / 2);
+}
+// shared-memory copy of the tables (8-byte units): [D][entries] the direction operators, then [NP] l(+-1),
+// and for the lifting the direction operators again, times mu
 template <int D, int NP>
 __host__ __device__ constexpr int fx_tab_smem() {
-  return D * NP * (NP + 2) + 2 * NP;
+  return D * fx_entries<NP>() + NP;
 }
 template <int D, int NP>
 __host__ __device__ constexpr int fx_tab_lift_smem() {
-  return fx_tab_smem<D, NP>() + D * NP * (NP + 2);
+  return fx_tab_smem<D, NP>() + D * fx_entries<NP>();
 }
 template <int D, int NP, bool LIFT>
 __device__ __forceinline__ void fx_stage_tables(const NskFx& f, int2* tb) {
-  constexpr int W = NP + 2;
-  for (int x = threadIdx.x; x < D * NP * W; x += blockDim.x) {
-    const int k = x / (NP * W), r = x % (NP * W);
-    const int2 v = f.d[k][r / W][r % W];
+  constexpr int NE = fx_entries<NP>();
+  for (int x = threadIdx.x; x < D * NE; x += blockDim.x) {
+    const int2 v = f.d[x / NE][x % NE];
     tb[x] = v;
     if constexpr (LIFT) {  // the 58-bit entry times mu's 63-bit mantissa, back at 58 bits
       const long long q = __mul64hi(((long long)v.x << 29) + ((long long)v.y << 1), f.mum);
       tb[fx_tab_smem<D, NP>() + x] = make_int2((int)(q >> 28), (int)(q & 0xFFFFFFF));
     }
   }
-  for (int x = threadIdx.x; x < 2 * NP; x += blockDim.x) tb[D * NP * W + x] = f.l[x / NP][x % NP];
+  for (int x = threadIdx.x; x < NP; x += blockDim.x) tb[D * NE + x] = f.l[x];
 }
 
-// The NP sums of one line: x its nodal values, xp and xm its +1 and -1 face values, T the rows of
+// n entries of a table, 16 bytes at a time where the row starts so aligned
+template <int N, bool PAIRED>
+__device__ __forceinline__ void fx_row(const int2* __restrict__ T, int2 (&t)[N]) {
+  if constexpr (PAIRED && N % 2 == 0) {
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+      const int4 q = *reinterpret_cast<const int4*>(T + j);
+      t[j] = make_int2(q.x, q.y);
+      t[j + 1] = make_int2(q.z, q.w);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; ++j) t[j] = T[j];
+  }
+}
+
+// The NP sums of one line: x its nodal values, xp and xm its +1 and -1 face values, T the entries of
 // the direction's operator; returns the line's E.
 template <int NP>
 __device__ __forceinline__ unsigned fx_line(const double (&x)[NP], const double xp, const double xm,
                                             const int2* __restrict__ T, long long (&acc)[NP]) {
-  constexpr int W = NP + 2;
+  constexpr int W = NP + 2, H = W / 2, HP = NP / 2;
   unsigned m = kFxMin;
 #pragma unroll
   for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
   m = max(max(m, fx_mag(xp)), fx_mag(xm));
   const unsigned E = m | 0xFFFFFu;
-  FxVal v[W];
+  FxVal sm[W - H], df[H];
 #pragma unroll
-  for (int j = 0; j < NP; ++j) v[j] = fx_val(x[j], E);
-  v[NP] = fx_val(xp, E);
-  v[NP + 1] = fx_val(xm, E);
+  for (int j = 0; j < H; ++j) {
+    const FxVal a = fx_val(j == 0 ? xm : x[j == 0 ? 0 : j - 1], E);
+    const FxVal b = fx_val(j == 0 ? xp : x[j == 0 ? 0 : NP - j], E);
+    sm[j] = FxVal{a.h + b.h, a.l + b.l};
+    df[j] = FxVal{a.h - b.h, a.l - b.l};
+  }
+  if constexpr (W % 2) sm[H] = fx_val(x[NP / 2], E);
 #pragma unroll
-  for (int i = 0; i < NP; ++i) {
+  for (int i = 0; i < HP; ++i) {
+    int2 t[W];
+    fx_row<W, W % 2 == 0>(T + i * W, t);
+    FxAcc a, b;
+    a.clear();
+    b.clear();
+#pragma unroll
+    for (int j = 0; j < H; ++j) a.mac(df[j], t[j]);
+#pragma unroll
+    for (int j = 0; j < W - H; ++j) b.mac(sm[j], t[H + j]);
+    const long long sa = a.sum(), sb = b.sum();
+    acc[i] = sa + sb;
+    acc[NP - 1 - i] = sa - sb;
+  }
+  if constexpr (NP % 2) {
     FxAcc a;
     a.clear();
-    if constexpr (W % 2 == 0) {  // rows start 16-byte aligned
 #pragma unroll
-      for (int j = 0; j < W; j += 2) {
-        const int4 t = *reinterpret_cast<const int4*>(T + i * W + j);
-        a.mac(v[j], make_int2(t.x, t.y));
-        a.mac(v[j + 1], make_int2(t.z, t.w));
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < W; ++j) a.mac(v[j], T[i * W + j]);
-    }
-    acc[i] = a.sum();
+    for (int j = 0; j < H; ++j) a.mac(df[j], T[HP * W + j]);
+    acc[HP] = a.sum();
   }
   return E;
 }
 
-// both face values of one line: x its nodal values, Tm and Tp the interpolation weights at -1 and
-// +1 (biased exponent et)
+// both face values of one line as sums at the returned exponent: x its nodal values, T the entries of
+// l(+-1) (biased exponent et)
 template <int NP>
-__device__ __forceinline__ void fx_ends(const double (&x)[NP], const int2* __restrict__ Tm,
-                                        const int2* __restrict__ Tp, const int et, double& om, double& op) {
+__device__ __forceinline__ int fx_ends_sum(const double (&x)[NP], const int2* __restrict__ T, const int et,
+                                           long long& om, long long& op) {
+  constexpr int H = NP / 2;
   unsigned m = kFxMin;
 #pragma unroll
   for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
@@ -211,28 +244,32 @@ __device__ __forceinline__ void fx_ends(const double (&x)[NP], const int2* __res
   a.clear();
   b.clear();
 #pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    const FxVal v = fx_val(x[j], E);
-    a.mac(v, Tm[j]);
-    b.mac(v, Tp[j]);
+  for (int j = 0; j < H; ++j) {
+    const FxVal u = fx_val(x[j], E), v = fx_val(x[NP - 1 - j], E);
+    a.mac(FxVal{u.h + v.h, u.l + v.l}, T[j]);
+    b.mac(FxVal{u.h - v.h, u.l - v.l}, T[NP - H + j]);
   }
-  const int e = fx_exp(E, et);
-  om = fx_out<false>(a.sum(), e);
-  op = fx_out<false>(b.sum(), e);
+  if constexpr (NP % 2) a.mac(fx_val(x[H], E), T[H]);
+  const long long sa = a.sum(), sb = b.sum();
+  op = sa + sb;
+  om = sa - sb;
+  return fx_exp(E, et);
 }
-
-// one face value of a line (weights T), the same value as fx_ends gives
 template <int NP>
-__device__ __forceinline__ double fx_end(const double (&x)[NP], const int2* __restrict__ T, const int et) {
-  unsigned m = kFxMin;
-#pragma unroll
-  for (int j = 0; j < NP; ++j) m = max(m, fx_mag(x[j]));
-  const unsigned E = m | 0xFFFFFu;
-  FxAcc a;
-  a.clear();
-#pragma unroll
-  for (int j = 0; j < NP; ++j) a.mac(fx_val(x[j], E), T[j]);
-  return fx_out<false>(a.sum(), fx_exp(E, et));
+__device__ __forceinline__ void fx_ends(const double (&x)[NP], const int2* __restrict__ T, const int et, double& om,
+                                        double& op) {
+  long long m, p;
+  const int e = fx_ends_sum<NP>(x, T, et, m, p);
+  om = fx_out<false>(m, e);
+  op = fx_out<false>(p, e);
+}
+// one of them (+1 when plus)
+template <int NP>
+__device__ __forceinline__ double fx_end(const double (&x)[NP], const int2* __restrict__ T, const int et,
+                                         const bool plus) {
+  long long m, p;
+  const int e = fx_ends_sum<NP>(x, T, et, m, p);
+  return fx_out<false>(plus ? p : m, e);
 }
 
 }  // namespace nsk

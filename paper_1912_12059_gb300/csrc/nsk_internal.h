@@ -41,10 +41,15 @@ struct NskTab {
 // The FP64 operator's matrices in the two-limb fixed-point form of nsk_fx.cuh (.x the signed high
 // limb, .y the low one), with the biased exponents of their scales.
 struct NskFx {
-  // row i of direction k: (2/h_k) dvol[i][j] (j < np), then the +1 and -1 faces' surface entries of
-  // a doubled face value: -lpk[i] / 2 and lmk[i] / 2
-  int2 d[3][NSK_MAXNP][NSK_MAXNP + 2];
-  int2 l[2][NSK_MAXNP];  // l_j(-1), l_j(+1)
+  // Direction k's operator on the np + 2 values g = (-1 face, nodes, +1 face) of a line, doubled face
+  // values: centro-antisymmetric, T[n-1-i][W-1-j] = -T[i][j] (n = np rows, W = np + 2). For each row pair i <
+  // np / 2: the W / 2 entries (T[i][j] - T[i][W-1-j]) / 2 of the differences g_j - g_(W-1-j), then the
+  // W - W / 2 entries (T[i][j] + T[i][W-1-j]) / 2 of the sums (the middle value's entry last when W is
+  // odd); for an odd np then the W / 2 difference entries of the middle row.
+  int2 d[3][4 * NSK_MAXNP];
+  // l(+-1): the np - np / 2 entries (l_j(+1) + l_(np-1-j)(+1)) / 2 of the sums of a line's node pairs (the
+  // middle node's entry last when np is odd), then np / 2 entries (l_j(+1) - l_(np-1-j)(+1)) / 2 of the differences
+  int2 l[NSK_MAXNP];
   long long mum;         // mu = mum 2^(mue - 63), 2^62 <= mum < 2^63 (0: mu = 0)
   int ed[3], el, mue;
 };

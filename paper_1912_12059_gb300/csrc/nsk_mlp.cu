@@ -46,6 +46,7 @@ extern "C" int nsk_gemm_bf16(const void* A, const void* B, int M, int N, int K, 
   if ((epilogue == nsk::tc::EPI_GELU || epilogue == nsk::tc::EPI_DGELU) && !hout) return NSK_ERR_ARG;
   if (epilogue == nsk::tc::EPI_DGELU && !zin) return NSK_ERR_ARG;
   nsk::tc::GemmArgs a;
+  memset(&a, 0, sizeof(a));
   a.A = (const __nv_bfloat16*)A;
   a.B = (const __nv_bfloat16*)B;
   a.M = M;
@@ -671,7 +672,7 @@ __global__ void __launch_bounds__(G * nsk::Shape<D, NP>::NPE)
 #pragma unroll
         for (int j = 0; j < NP; ++j) x[j] = sc[le * NPE + n0 + j * st];
         double om, op;
-        nsk::fx_ends<NP>(x, p.fx.l[0], p.fx.l[1], p.fx.el, om, op);
+        nsk::fx_ends<NP>(x, p.fx.l, p.fx.el, om, op);
         o[(size_t)(2 * k) * p.nfe + fn] = om;
         o[(size_t)(2 * k + 1) * p.nfe + fn] = op;
       }

@@ -4,10 +4,12 @@ the result, over line lengths, magnitudes, signs and exceptional values.
 
 Bound, derived from the representation before any run: a line's values lose less than 2^4 units of
 2^(E - 1023 - 61) each (the bits below the low limb; the shift and the one's complement of a negative
-value lie inside them), the matrix entries at most 2^3 units of 2^(es - 1023 - 61) (rounded to 2^4), each product's low-low part is below one unit of the sum and the sum of the cross
-products is floored once. With |value| < 2^62 units, row sums of the matrix below 2^62 units and W
-terms, the error is below 2^-64 (2^5 2^62 (W + 1)) + W + 1 < 10 (W + 1) units of the sum, and the
-rounding to FP64 adds half an ulp of the result."""
+value lie inside them); value pairs are added and subtracted exactly; the matrix entries (half sums and
+half differences) are off by at most 2^3 units of 2^(es - 1023 - 61) (rounded to 2^4). In units of the
+sum (2^64 of the product's): pairs below 2^63 times entry errors of 2^3, W entries: 4 W; pair errors
+below 2^5 times entries whose magnitudes add up to less than 2^62: 8; each low-low product below 2 units:
+2 W; two floors: 2. Together at most 10 (W + 1) units, and the rounding to FP64 adds half an ulp of the
+result."""
 import math
 from fractions import Fraction
 
@@ -44,17 +46,26 @@ def _val(x, E):
     return _s32((v >> 32) ^ s), ((v & M32) ^ s) >> 4
 
 
-def _line(xs, row):
-    """(sum, E): the sum of the row's products at the line's exponent."""
+def _line(xs, row, es):
+    """(sum, E): the row's sum at the line's exponent, from the sums and differences of value pairs."""
     E = max([100 << 20] + [_words(x)[0] & 0x7FFFFFFF for x in xs]) | 0xFFFFF
-    hh = cr = 0
-    for x, (th, tl) in zip(xs, row):
-        h, l = _val(x, E)
-        assert abs(h) <= 1 << 30 and 0 <= l < 1 << 28 and abs(th) <= 1 << 30 and 0 <= tl < 1 << 28
-        hh += h * th
-        cr += h * tl + l * th
-    assert abs(hh) < 1 << 62 and abs(cr) < 1 << 62
-    return hh + (cr >> 28), E
+    v = [_val(x, E) for x in xs]
+    W, total = len(xs), 0
+    for sign in (-1, 1):
+        hh = cr = 0
+        for j in range(W // 2 + (W % 2 if sign > 0 else 0)):
+            k = W - 1 - j
+            if j == k:
+                (h, low), (th, tl) = v[j], _entry(row[j], es)
+            else:
+                h, low = v[j][0] + sign * v[k][0], v[j][1] + sign * v[k][1]
+                th, tl = _entry((row[j] + sign * row[k]) / 2, es)
+            assert -(1 << 31) <= h < 1 << 31 and abs(low) < 1 << 29 and abs(th) <= 1 << 30 and 0 <= tl < 1 << 28
+            hh += h * th
+            cr += h * tl + low * th
+        assert abs(hh) < 1 << 62 and abs(cr) < 1 << 62
+        total += hh + (cr >> 28)
+    return total, E
 
 
 def _out(a, e):
@@ -73,7 +84,7 @@ def _out(a, e):
 
 
 def _contract(xs, row, es):
-    a, E = _line(xs, [_entry(t, es) for t in row])
+    a, E = _line(xs, row, es)
     ex = E >> 20
     return _out(a, ex + es + (65536 if ex >= 0x7FF else -65536 if ex <= 100 else 0)), ex
 
