@@ -53,6 +53,7 @@ struct GemmArgs {
   int M, N, K, lda, ldb;
   int k_split;             // K per gridDim.y slice (multiple of kKC), or K
   int epi;
+  int nslice;              // columns per gridDim.y slice (resident kernel), 0: all
   const float* bias;       // [N] or NULL
   float* out;              // FP32 [M][ldo] (STORE, ATOMIC) or z [M][ldo] (GELU, optional)
   int ldo;
@@ -463,12 +464,32 @@ __device__ __forceinline__ void epilogue_chunk_rb(const GemmArgs& a, const int r
   }
 }
 
-// gridDim.y > 1: the CTAs of row y hold the 64 columns (rows of B) from 64 y on (the last row's may
-// be 16 to 48), so that a batch of few row tiles still fills the SMs; a column's sum does not depend
-// on the split. a.N then is the whole matrix's.
+// One warp's lanes' place in a sweep of 16-byte chunks over rows of kc chunks by kRbThreads threads: the
+// row and the chunk advance by fixed steps, without a division per chunk.
+struct ChunkWalk {
+  int r, j, dr, dj, kc;
+  __device__ __forceinline__ explicit ChunkWalk(int kc_) : kc(kc_) {
+    r = threadIdx.x / kc;
+    j = threadIdx.x % kc;
+    dr = kRbThreads / kc;
+    dj = kRbThreads % kc;
+  }
+  __device__ __forceinline__ void next() {
+    r += dr;
+    j += dj;
+    if (j >= kc) {
+      j -= kc;
+      ++r;
+    }
+  }
+};
+
+// nslice > 0: the CTAs of row y hold the nslice columns (rows of B) from nslice y on (the last row's may
+// be fewer, a multiple of 16), so that a batch of few row tiles still fills the SMs; a column's sum does
+// not depend on the split.
 __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  const int K = a.K, n0 = blockIdx.y * 64, N = gridDim.y > 1 ? min(64, a.N - n0) : a.N;
+  const int K = a.K, n0 = blockIdx.y * a.nslice, N = a.nslice ? min(a.nslice, a.N - n0) : a.N;
   unsigned char* sB = smem;
   unsigned char* sA = smem + rb_b_bytes(N, K);
   float* stage = reinterpret_cast<float*>(sA + kBM * K * 2) + (threadIdx.x >> 5) * kStage;
@@ -493,10 +514,8 @@ __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) 
   }
   // resident B
   const uint32_t sBa = smem_u32(sB), sAa = smem_u32(sA);
-  for (int idx = threadIdx.x; idx < N * kc; idx += kRbThreads) {
-    const int r = idx / kc, j = idx % kc;
-    cp_async16(sBa + core_off_k(r, j * 8, K), a.B + (size_t)(n0 + r) * a.ldb + j * 8, 16);
-  }
+  for (ChunkWalk w(kc); w.r < N; w.next())
+    cp_async16(sBa + core_off_k(w.r, w.j * 8, K), a.B + (size_t)(n0 + w.r) * a.ldb + w.j * 8, 16);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
@@ -516,11 +535,10 @@ __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) 
     }
     if (have) {
       const int m0 = t * kBM;
-      for (int idx = threadIdx.x; idx < kBM * kc; idx += kRbThreads) {
-        const int r = idx / kc, j = idx % kc;
-        const bool v = m0 + r < a.M;
-        cp_async16(sAa + core_off_k(r, j * 8, K), v ? (const void*)(a.A + (size_t)(m0 + r) * a.lda + j * 8)
-                                                    : (const void*)a.A, v ? 16 : 0);
+      for (ChunkWalk w(kc); w.r < kBM; w.next()) {
+        const bool v = m0 + w.r < a.M;
+        cp_async16(sAa + core_off_k(w.r, w.j * 8, K), v ? (const void*)(a.A + (size_t)(m0 + w.r) * a.lda + w.j * 8)
+                                                        : (const void*)a.A, v ? 16 : 0);
       }
       asm volatile("cp.async.wait_all;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1459,12 +1477,15 @@ inline int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   const bool resident = a.epi != EPI_ATOMIC && a.k_split >= a.K && a.K <= 256 && aligned;
   // few row tiles: 64-column slices fill the SMs (4096 rows of a 256 x 256 layer: 128 blocks instead of
   // 32, each with a quarter of the epilogue); many: one block per SM holds the whole B
-  const int ny = (a.N + 63) / 64;
-  if (resident && (ntiles * ny <= sms || a.N % 64)) {
-    int smem = rb_b_bytes(64, a.K) + kBM * a.K * 2 + kRbStageBytes;
+  if (resident && (ntiles * ((a.N + 63) / 64) <= sms || a.N % 64)) {
+    GemmArgs b = a;
+    b.nslice = 64;
+    while (b.nslice > 16 && ntiles * ((a.N + b.nslice / 2 - 1) / (b.nslice / 2)) <= sms) b.nslice /= 2;
+    const int ny = (a.N + b.nslice - 1) / b.nslice;
+    int smem = rb_b_bytes(b.nslice, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
     const int gx = (int)persistent_grid(ntiles, sms / ny > 0 ? sms / ny : 1);
-    k_gemm_tc_rb<<<dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s>>>(a);
+    k_gemm_tc_rb<<<dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s>>>(b);
   } else if (resident) {
     int smem = rb_b_bytes(a.N, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
