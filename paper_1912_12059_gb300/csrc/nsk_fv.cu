@@ -35,14 +35,17 @@ struct FvParams {
   double Vinv[NSK_MAXNP * NSK_MAXNP];  // nodal values -> orthonormal Legendre modes, [m][i]
   double Ub[2][3];                     // Dirichlet states outside x = lo (0) and x = hi (1)
   double upper, lower;                 // indicator thresholds (log10)
-  double dx;                           // sub-cell width h / (N+1)
+  double dx, idx;                      // sub-cell width h / (N+1) and its inverse
   int dirichlet;
 };
 
-// one-dimensional state helpers ----------------------------------------------------------
+// One-dimensional state helpers. A phase of the small-mesh kernel lasts as long as its longest serial
+// chain, and an FP64 division or square root is a chain of about ten FP64 operations at one per 64 clocks
+// of a scheduler; quotients therefore go through the integer reciprocal and roots through the integer
+// root (rcp_nr, sqrt_nr).
 __device__ __forceinline__ void prim(const double* U, double* P) {
   P[0] = U[0];
-  P[1] = U[1] / U[0];
+  P[1] = U[1] * rcp_nr(U[0]);
   P[2] = U[2];
 }
 __device__ __forceinline__ void cons(const double* P, double* U) {
@@ -66,12 +69,15 @@ __device__ __forceinline__ bool bad(double rho) { return !rho_ok(rho); }
 // p_alpha (Davis speeds); c has no convective flux (LF adds its jump only with c_diss).
 __device__ void numflux(const NskParams& p, const double* L, const double* R, double* F, int& eflag) {
   double pl, dl, pr, dr;
-  eos_both64(p, L[0], pl, dl);
-  eos_both64(p, R[0], pr, dr);
+  // one reciprocal per side: d = 1/(rho (3 - rho)) gives 1/rho = (3 - rho) d and 1/(3 - rho) = rho d
+  const double gl = 3.0 - L[0], gr = 3.0 - R[0];
+  const double ddl = rcp_nr(L[0] * gl), ddr = rcp_nr(R[0] * gr);
+  Eos<double>::both_q(p, L[0], L[0] * ddl, pl, dl);
+  Eos<double>::both_q(p, R[0], R[0] * ddr, pr, dr);
   if (!sound_ok(dl) || !sound_ok(dr)) eflag |= NSK_EBIT_SOUND;
   if (bad(L[0]) || bad(R[0])) eflag |= NSK_EBIT_RHO;
-  const double ul = L[1] / L[0], ur = R[1] / R[0];
-  const double al = sqrt(dl), ar = sqrt(dr);
+  const double ul = L[1] * (gl * ddl), ur = R[1] * (gr * ddr);
+  const double al = sqrt_nr(dl), ar = sqrt_nr(dr);
   const double fl[2] = {L[1], L[1] * ul + pl}, fr[2] = {R[1], R[1] * ur + pr};
   if (p.flux == NSK_FLUX_HLLC) {
     const double SL = fmin(ul - al, ur - ar), SR = fmax(ul + al, ur + ar);
@@ -87,10 +93,10 @@ __device__ void numflux(const NskParams& p, const double* L, const double* R, do
       return;
     }
     const double wl = L[0] * (SL - ul), wr = R[0] * (SR - ur);
-    const double Ss = (pr - pl + wl * ul - wr * ur) / (wl - wr);
+    const double Ss = (pl - pr + wr * ur - wl * ul) * rcp_nr(wr - wl);
     const bool left = Ss >= 0.0;
     const double SK = left ? SL : SR, rk = left ? L[0] : R[0], mk = left ? L[1] : R[1];
-    const double coef = (left ? wl : wr) / (SK - Ss);
+    const double coef = (left ? -wl : wr) * rcp_nr(left ? Ss - SL : SR - Ss);
     F[0] = (left ? fl[0] : fr[0]) + SK * (coef - rk);
     F[1] = (left ? fl[1] : fr[1]) + SK * (coef * Ss - mk);
     return;
@@ -192,33 +198,33 @@ __device__ __forceinline__ void fv_faces_body(const NskParams& p, const FvParams
     if (bad(c[0])) eflag |= NSK_EBIT_RHO;
     prim(c, P[j]);
   }
-  double Pn[2][3], dn[2];  // the value beyond each element face, and its distance from the end cell's centre
+  double Pn[2][3], idn[2];  // the value beyond each element face, and 1 / its distance from the end cell's centre
 #pragma unroll
   for (int sd = 0; sd < 2; ++sd) {
     const long long en = nbr(p, f, e, sd);
     if (en < 0) {
       prim(f.Ub[sd], Pn[sd]);
-      dn[sd] = 0.5 * f.dx;
+      idn[sd] = 2.0 * f.idx;
     } else if (flags[en]) {
       const int jn = sd ? 0 : NP - 1;
       const double c[3] = {U[en * NP + jn], U[(size_t)p.nne + en * NP + jn], U[2 * (size_t)p.nne + en * NP + jn]};
       prim(c, Pn[sd]);
-      dn[sd] = f.dx;
+      idn[sd] = f.idx;
     } else {
       double c[3];
 #pragma unroll
       for (int v = 0; v < 3; ++v) c[v] = dg_trace<NP>(p, U, en, v, sd ? 0 : 1);
       prim(c, Pn[sd]);
-      dn[sd] = 0.5 * f.dx;
+      idn[sd] = 2.0 * f.idx;
     }
   }
-  const double idx = 1.0 / f.dx;
+  const double idx = f.idx;
 #pragma unroll
   for (int j = 0; j < NP; ++j)
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      const double lq = j > 0 ? (P[j][q] - P[j - 1][q]) * idx : (P[0][q] - Pn[0][q]) / dn[0];
-      const double rq = j < NP - 1 ? (P[j + 1][q] - P[j][q]) * idx : (Pn[1][q] - P[NP - 1][q]) / dn[1];
+      const double lq = j > 0 ? (P[j][q] - P[j - 1][q]) * idx : (P[0][q] - Pn[0][q]) * idn[0];
+      const double rq = j < NP - 1 ? (P[j + 1][q] - P[j][q]) * idx : (Pn[1][q] - P[NP - 1][q]) * idn[1];
       SL[(e * NP + j) * 3 + q] = minmod(lq, rq);
     }
   double Pl[3], Pr[3], Ul[3], Ur[3];
@@ -236,8 +242,8 @@ __device__ __forceinline__ void fv_faces_body(const NskParams& p, const FvParams
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    Gf[(e * 2 + 0) * 2 + q] = (P[0][1 + q] - Pn[0][1 + q]) / dn[0];
-    Gf[(e * 2 + 1) * 2 + q] = (Pn[1][1 + q] - P[NP - 1][1 + q]) / dn[1];
+    Gf[(e * 2 + 0) * 2 + q] = (P[0][1 + q] - Pn[0][1 + q]) * idn[0];
+    Gf[(e * 2 + 1) * 2 + q] = (Pn[1][1 + q] - P[NP - 1][1 + q]) * idn[1];
   }
   if (eflag) atomicOr(err, eflag);
 }
@@ -260,14 +266,14 @@ __device__ __forceinline__ void fv_lift_body(const NskParams& p, const FvParams&
   for (int sd = 0; sd < 2; ++sd) {
     const double* Ui = Uf + (e * 2 + sd) * 3;
     const double* Uo = outer(p, f, Uf, e, sd);
-    ws[sd][0] = 0.5 * (Ui[1] / Ui[0] + Uo[1] / Uo[0]);
+    ws[sd][0] = 0.5 * (Ui[1] * rcp_nr(Ui[0]) + Uo[1] * rcp_nr(Uo[0]));
     ws[sd][1] = 0.5 * (Ui[2] + Uo[2]);
   }
   double w[2][NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
     const double rho = U[e * NP + j];
-    w[0][j] = U[(size_t)p.nne + e * NP + j] / rho;
+    w[0][j] = U[(size_t)p.nne + e * NP + j] * rcp_nr(rho);
     w[1][j] = U[2 * (size_t)p.nne + e * NP + j];
   }
   double q[2][NP];
@@ -359,12 +365,12 @@ __device__ __forceinline__ void fv_update_body(const NskParams& p, const FvParam
     double F[3][NP], qc[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
-      const double rho = u[0][j], vel = u[1][j] / rho;
+      const double rho = u[0][j], g3 = 3.0 - rho, d = rcp_nr(rho * g3), vel = u[1][j] * (g3 * d);
       if (bad(rho)) eflag |= NSK_EBIT_RHO;
       const double qv = Q[e * NP + j];
       qc[j] = Q[(size_t)p.nne + e * NP + j];
       F[0][j] = u[1][j];
-      F[1][j] = fma(u[1][j], vel, eos_pa64(p, rho)) - (4.0 / 3.0) * t.mu * qv;
+      F[1][j] = fma(u[1][j], vel, Eos<double>::pa_q(p, rho, rho * d)) - (4.0 / 3.0) * t.mu * qv;
       F[2][j] = -t.kb * qc[j];
     }
 #pragma unroll
@@ -390,7 +396,7 @@ __device__ __forceinline__ void fv_update_body(const NskParams& p, const FvParam
 #pragma unroll
       for (int q = 0; q < 3; ++q) s[j][q] = SL[(e * NP + j) * 3 + q];
     }
-    const double idx = 1.0 / f.dx;
+    const double idx = f.idx;
     double Fs[NP + 1][3], gc[NP + 1];  // sub-cell face fluxes, c_x on the sub-cell faces
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
@@ -479,35 +485,35 @@ __device__ __forceinline__ void fv_faces_group(const NskParams& p, const FvParam
     prim(c, P);
   }
   // the value beyond the element's face on the lane's side (lane 0: side 0, lane NP - 1: side 1)
-  double Pn[3] = {0.0, 0.0, 0.0}, dn = 1.0;
+  double Pn[3] = {0.0, 0.0, 0.0}, idn = 1.0;
   const int sd = j == 0 ? 0 : 1;
   if (active && (j == 0 || j == NP - 1)) {
     const long long en = nbr(p, f, e, sd);
     if (en < 0) {
       prim(f.Ub[sd], Pn);
-      dn = 0.5 * f.dx;
+      idn = 2.0 * f.idx;
     } else if (flags[en]) {
       const int jn = sd ? 0 : NP - 1;
       const double c[3] = {U[en * NP + jn], U[(size_t)p.nne + en * NP + jn], U[2 * (size_t)p.nne + en * NP + jn]};
       prim(c, Pn);
-      dn = f.dx;
+      idn = f.idx;
     } else {
       double c[3];
 #pragma unroll
       for (int v = 0; v < 3; ++v) c[v] = dg_trace<NP>(p, U, en, v, sd ? 0 : 1);
       prim(c, Pn);
-      dn = 0.5 * f.dx;
+      idn = 2.0 * f.idx;
     }
   }
   const int base = (threadIdx.x & 31) & ~(W - 1);
-  const double idx = 1.0 / f.dx;
+  const double idx = f.idx;
   double slope[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const double Pm = grp_get(P[q], base + (j > 0 ? j - 1 : 0), W);  // P[j - 1]
     const double Pp = grp_get(P[q], base + (j < NP - 1 ? j + 1 : j), W);  // P[j + 1]
-    const double lq = j > 0 ? (P[q] - Pm) * idx : (P[q] - Pn[q]) / dn;
-    const double rq = j < NP - 1 ? (Pp - P[q]) * idx : (Pn[q] - P[q]) / dn;
+    const double lq = j > 0 ? (P[q] - Pm) * idx : (P[q] - Pn[q]) * idn;
+    const double rq = j < NP - 1 ? (Pp - P[q]) * idx : (Pn[q] - P[q]) * idn;
     slope[q] = minmod(lq, rq);
     if (mine) SL[(e * NP + j) * 3 + q] = slope[q];
   }
@@ -520,7 +526,7 @@ __device__ __forceinline__ void fv_faces_group(const NskParams& p, const FvParam
     for (int v = 0; v < 3; ++v) Uf[(e * 2 + sd) * 3 + v] = Uo[v];
 #pragma unroll
     for (int q = 0; q < 2; ++q)
-      Gf[(e * 2 + sd) * 2 + q] = j == 0 ? (P[1 + q] - Pn[1 + q]) / dn : (Pn[1 + q] - P[1 + q]) / dn;
+      Gf[(e * 2 + sd) * 2 + q] = j == 0 ? (P[1 + q] - Pn[1 + q]) * idn : (Pn[1 + q] - P[1 + q]) * idn;
   }
   if (eflag) atomicOr(err, eflag);
 }
@@ -541,13 +547,13 @@ __device__ __forceinline__ void fv_lift_group(const NskParams& p, const FvParams
     for (int sd = 0; sd < 2; ++sd) {
       const double* Ui = Uf + (e * 2 + sd) * 3;
       const double* Uo = outer(p, f, Uf, e, sd);
-      ws[sd][0] = 0.5 * (Ui[1] / Ui[0] + Uo[1] / Uo[0]);
+      ws[sd][0] = 0.5 * (Ui[1] * rcp_nr(Ui[0]) + Uo[1] * rcp_nr(Uo[0]));
       ws[sd][1] = 0.5 * (Ui[2] + Uo[2]);
     }
   }
   if (mine) {
     const double rho = U[e * NP + j];
-    w[0] = U[(size_t)p.nne + e * NP + j] / rho;
+    w[0] = U[(size_t)p.nne + e * NP + j] * rcp_nr(rho);
     w[1] = U[2 * (size_t)p.nne + e * NP + j];
   }
   double q[2];
@@ -609,12 +615,12 @@ __device__ __forceinline__ void fv_update_group(const NskParams& p, const FvPara
     }
     double F[3], qc;
     {
-      const double rho = u[0], vel = u[1] / rho;
+      const double rho = u[0], g3 = 3.0 - rho, d = rcp_nr(rho * g3), vel = u[1] * (g3 * d);
       if (mine && bad(rho)) eflag |= NSK_EBIT_RHO;
       const double qv = mine ? Q[e * NP + j] : 0.0;
       qc = mine ? Q[(size_t)p.nne + e * NP + j] : 0.0;
       F[0] = u[1];
-      F[1] = fma(u[1], vel, eos_pa64(p, rho)) - (4.0 / 3.0) * t.mu * qv;
+      F[1] = fma(u[1], vel, Eos<double>::pa_q(p, rho, rho * d)) - (4.0 / 3.0) * t.mu * qv;
       F[2] = -t.kb * qc;
     }
 #pragma unroll
@@ -632,7 +638,7 @@ __device__ __forceinline__ void fv_update_group(const NskParams& p, const FvPara
     if (mine)
 #pragma unroll
       for (int q = 0; q < 3; ++q) s[q] = SL[(e * NP + j) * 3 + q];
-    const double idx = 1.0 / f.dx;
+    const double idx = f.idx;
     double Pm[3], sm[3];  // sub-cell j - 1
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -734,6 +740,41 @@ __global__ void __launch_bounds__(128)
 // sub-cell element's internal HLLC solves run side by side instead of one after another, and the
 // update's groups evaluate the element-face fluxes themselves, so a stage has three phases.
 constexpr int kCoopMaxE = 4096;
+
+// Grid barrier of that launch on one counter that only grows (zero at the launch): a block adds one and
+// waits until the count reaches the next multiple of the grid. One atomic and one read of the counter lie
+// between the last arrival and the release; a counter reset and a separate generation word (and a read of
+// the error word) cost three more trips to the L2 per barrier, 16 barriers a step. A block that waits
+// longer than timeout_ns sets NSK_EBIT_TIMEOUT and the counter's top bit, and every block then returns false.
+constexpr unsigned long long kBarAbort = 1ull << 63;
+__device__ __forceinline__ bool coop_barrier(unsigned long long* bar, int* err, const unsigned long long timeout_ns) {
+  bool ok = true;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long seen = atomicAdd(bar, 1ull), n = gridDim.x;
+    if (seen & kBarAbort) {
+      ok = false;
+    } else {
+      const unsigned long long target = (seen / n + 1) * n;
+      volatile unsigned long long* v = bar;
+      unsigned long long c = *v;
+      const unsigned long long t0 = c < target ? global_ns() : 0;
+      while (c < target) {
+        if (global_ns() - t0 > timeout_ns) {
+          atomicOr(err, NSK_EBIT_TIMEOUT);
+          atomicOr(bar, kBarAbort);
+          ok = false;
+          break;
+        }
+        c = *v;
+      }
+      if (c & kBarAbort) ok = false;
+    }
+    __threadfence();
+  }
+  return !__syncthreads_or(!ok);
+}
 struct LsrkCoef {
   double A[5], B[5];
 };
@@ -745,7 +786,7 @@ __global__ void __launch_bounds__(32) k_fv_coop(const NskParams p, const FvParam
                                                 double* __restrict__ Gf, double* __restrict__ SL,
                                                 double* __restrict__ Q, const int nsteps,
                                                 const int switching, const double dt, const LsrkCoef rk,
-                                                unsigned* __restrict__ bar, int* __restrict__ err,
+                                                unsigned long long* __restrict__ bar, int* __restrict__ err,
                                                 const unsigned long long timeout_ns) {
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   // faces and update: the first half of the blocks takes the DG elements, the second the FV ones
@@ -760,18 +801,18 @@ __global__ void __launch_bounds__(32) k_fv_coop(const NskParams p, const FvParam
   for (int step = 0; step < nsteps; ++step) {
     if (switching) {
       for (long long e = first; e < p.E; e += stride) fv_switch_body<NP>(p, f, U, flags, ind, e);
-      if (!grid_barrier(bar, err, timeout_ns)) return;
+      if (!coop_barrier(bar, err, timeout_ns)) return;
     }
     for (int st = 0; st < 5; ++st) {
       for (long long eb = rgfirst; eb < p.E; eb += rgstride)
         fv_faces_group<NP>(p, f, U, flags, Uf, Gf, SL, err, eb + grp, j, role);
-      if (!grid_barrier(bar, err, timeout_ns)) return;
+      if (!coop_barrier(bar, err, timeout_ns)) return;
       for (long long eb = gfirst; eb < p.E; eb += gstride) fv_lift_group<NP>(p, f, U, flags, Uf, Q, Gf, eb + grp, j);
-      if (!grid_barrier(bar, err, timeout_ns)) return;
+      if (!coop_barrier(bar, err, timeout_ns)) return;
       // (the element-face fluxes are evaluated by the update's lane groups: no face phase)
       for (long long eb = rgfirst; eb < p.E; eb += rgstride)
         fv_update_group<NP>(p, f, U, K, flags, Uf, Gf, SL, Q, rk.A[st], rk.B[st], dt, err, eb + grp, j, role);
-      if (!grid_barrier(bar, err, timeout_ns)) return;
+      if (!coop_barrier(bar, err, timeout_ns)) return;
     }
   }
 }
@@ -828,7 +869,7 @@ int launch_coop_t(const NskParams& p, const FvParams& f, const FvBuffers& fb, co
   // a barrier that timed out in an earlier launch may have left its arrival count behind
   if (cudaMemsetAsync(fb.bar, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return NSK_ERR_CUDA;
   if (cudaLaunchKernelEx(&cfg, kern, p, f, (double*)b.U, (double*)b.K, fb.flags, fb.ind, fb.Uf, fb.Gf, fb.SL,
-                         (double*)b.Q, nsteps, switching, dt, rk, fb.bar, b.err, timeout_ns) != cudaSuccess)
+                         (double*)b.Q, nsteps, switching, dt, rk, (unsigned long long*)fb.bar, b.err, timeout_ns) != cudaSuccess)
     return NSK_ERR_CUDA;
   return 1;
 }
@@ -953,5 +994,6 @@ int nsk_fv_fill_params(void* fvp, int np, const double* xi, const double* gauss_
   f.upper = upper;
   f.lower = lower;
   f.dx = h / np;
+  f.idx = 1.0 / f.dx;
   return NSK_OK;
 }
