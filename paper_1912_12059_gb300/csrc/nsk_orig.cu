@@ -17,9 +17,26 @@
 namespace nsk {
 namespace orig {
 
+// Where the contractions are in integers (nsk_fx.cuh: 2D and 3D, lines of 3 nodes or more) the kernels
+// below keep doubled face values (the central sums, 2 F*), as the integer operator expects; K then holds
+// the register over dt. The second lifting's face fluxes interpolate 13 values per face node and were 40 %
+// of a stage; a thread there forms both ends of one line.
+
 // plain VdW pressure with q = 1/(3 - rho): p = 8 T rho q - 3 rho^2
 __device__ __forceinline__ double pressure_q(const NskParams& p, double rho, double q) {
-  return fma(p.t8 * rho, q, -3.0 * rho * rho);
+  return rho * fma(-3.0, rho, p.t8 * q);
+}
+
+template <int D, int NP>
+__host__ __device__ constexpr int tab_orig() {
+  return tab_smem_r<double, D, NP>();
+}
+template <int D, int NP>
+__device__ __forceinline__ void tables_orig(const NskParams& p, double* tb) {
+  if constexpr (fx_on<double, D, NP>())
+    fx_stage_tables<D, NP, false>(p.fx, reinterpret_cast<int2*>(tb));
+  else
+    stage_tables<double, D, NP>(p.td, tb);
 }
 
 template <int D, int NP, int G>
@@ -27,6 +44,15 @@ __host__ __device__ constexpr int lift2_work() {
   using S = Shape<D, NP>;
   return (G * D * S::NPE + G * S::NF * S::NFN) > (G * (S::NQ + 1) * S::NPE) ? (G * D * S::NPE + G * S::NF * S::NFN)
                                                                            : (G * (S::NQ + 1) * S::NPE);
+}
+
+// a[k s] for a runtime k < D through selects over compile-time indices (the array stays in registers)
+template <int D>
+__device__ __forceinline__ double pick(const double* a, const int s, const int k) {
+  double r = a[0];
+  if constexpr (D > 1) r = k == 1 ? a[s] : r;
+  if constexpr (D > 2) r = k == 2 ? a[2 * s] : r;
+  return r;
 }
 
 // (tau + tau^K)_{.k}, momentum components, from rho, the gradients q (q[k*(d+1)+a] = d v_a/dx_k,
@@ -42,13 +68,11 @@ __device__ __forceinline__ void visc_kort(const NskParams& p, const int k, const
     g2 = fma(q[a * NW + D], q[a * NW + D], g2);
   }
   const double iso = p.kappa * fma(rho, lap, 0.5 * g2);
+  const double kg = -(p.kappa * pick<D>(q + D, NW, k));
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    double tau = q[k * NW + a] + q[a * NW + k];
-    if (a == k) tau = fma(-2.0 / 3.0, div, tau);
-    double tk = -(p.kappa * q[a * NW + D]) * q[k * NW + D];
-    if (a == k) tk += iso;
-    f[a] = fma(p.mu, tau, tk);
+    const double tau = pick<D>(q + a, NW, k) + pick<D>(q + a * NW, 1, k);
+    f[a] = fma(p.mu, a == k ? fma(-2.0 / 3.0, div, tau) : tau, fma(kg, q[a * NW + D], a == k ? iso : 0.0));
   }
 }
 
@@ -66,34 +90,61 @@ __device__ __forceinline__ void lift2_group(const NskParams& p, const double* __
   constexpr int NPE = S::NPE, NFN = S::NFN, NW = S::NW, NF = S::NF, NQ = S::NQ;
   double* sg = sm;                    // [G][D][NPE] grad rho at the nodes
   double* sgs = sm + G * D * NPE;     // [G][NF][NFN] central (grad rho)_k on the faces of direction k
-  double* tb = sm + lift2_work<D, NP, G>();
+  double* tb = sm + ((lift2_work<D, NP, G>() + 1) & ~1);
   const auto& t = p.td;
+  constexpr bool FX = fx_on<double, D, NP>();
   const int le = threadIdx.x / NPE, n = threadIdx.x % NPE;
   const int e = (int)e0 + le;
   const bool valid = le < G && e < p.E;
   const size_t nn = (size_t)p.nne;
   const int g = e * NPE + n;
 
-  stage_tables<double, D, NP>(t, tb);
+  tables_orig<D, NP>(p, tb);
   double q[NQ], rho = 0.0;
   if (valid) {
     rho = U[g];
 #pragma unroll
     for (int c = 0; c < NQ; ++c) q[c] = Q[c * nn + g];
 #pragma unroll
-    for (int k = 0; k < D; ++k) sg[(le * D + k) * NPE + n] = q[k * NW + D];
+    for (int k = 0; k < D; ++k) {
+      if constexpr (FX)
+        sg[fx_pos<NP>((le * D + k) * NFN + face_node<D, NP>(n, k), coord<NP>(n, k))] = q[k * NW + D];
+      else
+        sg[(le * D + k) * NPE + n] = q[k * NW + D];
+    }
     const ElemIdx ex = elem_idx<D>(p, e);
     for (int it = n; it < NF * NFN; it += NPE) {
       const int slot = it / NFN, fn = it % NFN, k = slot >> 1, s = slot & 1;
       const int en = nbr_of(p, ex, k, s ? 1 : -1);
       const double go = Gtr[(size_t)slot * p.nfe + (e * NFN + fn)];
       const double gn = Gtr[(size_t)(2 * k + 1 - s) * p.nfe + (en * NFN + fn)];
-      sgs[(le * NF + slot) * NFN + fn] = 0.5 * (go + gn);
+      sgs[(le * NF + slot) * NFN + fn] = FX ? go + gn : 0.5 * (go + gn);
     }
   }
   __syncthreads();
   double lap = 0.0;
-  if (valid) {
+  if constexpr (FX) {
+    if (valid) {  // the element's lines, one thread each (D NFN <= NPE for these shapes)
+      for (int L = n; L < D * NFN; L += NPE) {
+        const int k = L / NFN, fn = L % NFN, Lg = le * D * NFN + L;
+        double* fm = sgs + (le * NF + 2 * k) * NFN + fn;
+        double x[NP];
+        fx_load<NP>(sg, Lg, x);
+        long long acc[NP];
+        const unsigned E =
+            fx_line<NP>(x, fm[NFN], *fm, reinterpret_cast<const int2*>(tb) + k * fx_entries<NP>(), acc);
+        fx_store<NP>(sg, Lg, acc);
+        *fm = __hiloint2double(0, fx_exp(E, p.fx.ed[k]));
+      }
+    }
+    __syncthreads();
+    if (valid) {
+      double l1[1];
+      volume_sums_fx<D, NP, 1>(sg, sgs, le, n, l1);
+      lap = -l1[0];
+      Q2[g] = lap;
+    }
+  } else if (valid) {
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       const int i = coord<NP>(n, k), fn = face_node<D, NP>(n, k);
@@ -115,7 +166,31 @@ __device__ __forceinline__ void lift2_group(const NskParams& p, const double* __
     sq[(le * (NQ + 1) + NQ) * NPE + n] = lap;
   }
   __syncthreads();
-  if (valid) {
+  if constexpr (FX) {
+    if (valid) {
+      const size_t pl = (size_t)NF * p.nfe;
+      for (int it = n; it < D * NFN; it += NPE) {
+        const int k = it / NFN, fn = it % NFN;
+        const int n0 = line_base<D, NP>(fn, k), st = node_stride<NP>(k);
+        double tm[NQ + 1], tp[NQ + 1];
+#pragma unroll
+        for (int c = 0; c <= NQ; ++c) {
+          double x[NP];
+#pragma unroll
+          for (int j = 0; j < NP; ++j) x[j] = sq[(le * (NQ + 1) + c) * NPE + n0 + j * st];
+          fx_ends<NP>(x, p.fx.l, p.fx.el, tm[c], tp[c]);
+        }
+        const size_t off = (size_t)(2 * k) * p.nfe + (e * NFN + fn);
+        double f[D];
+        visc_kort<D>(p, k, Utr[off], tm, tm[NQ], f);
+#pragma unroll
+        for (int a = 0; a < D; ++a) FVtr[off + a * pl] = f[a];
+        visc_kort<D>(p, k, Utr[off + p.nfe], tp, tp[NQ], f);
+#pragma unroll
+        for (int a = 0; a < D; ++a) FVtr[off + p.nfe + a * pl] = f[a];
+      }
+    }
+  } else if (valid) {
     const size_t pl = (size_t)NF * p.nfe;
     for (int it = n; it < NF * NFN; it += NPE) {
       const int slot = it / NFN, fn = it % NFN, k = slot >> 1;
@@ -170,11 +245,13 @@ __device__ __forceinline__ void face_at(const NskParams& p, const double* __rest
   const double mL = comp1<D>(UL, k), mR = comp1<D>(UR, k);
   const double vl = mL * il, vr = mR * ir;
   const double fnn = fma(mL, vl, pl) + fma(mR, vr, pr);
-  F[0] = 0.5 * (mL + mR);
+  constexpr bool FX = fx_on<double, D, NP>();  // 2 F*
+  F[0] = FX ? mL + mR : 0.5 * (mL + mR);
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     const double sum = (a == k) ? fnn : fma(vl, UL[1 + a], vr * UR[1 + a]);
-    F[1 + a] = fma(0.5, sum, -(0.5 * (vL[a * ps] + vR[a * ps])));
+    const double dif = sum - (vL[a * ps] + vR[a * ps]);
+    F[1 + a] = FX ? dif : 0.5 * dif;
   }
   double* o = Fstar + (size_t)k * p.nfe + (eL * NFN + fn);
 #pragma unroll
@@ -184,7 +261,7 @@ __device__ __forceinline__ void face_at(const NskParams& p, const double* __rest
 template <int D, int NP, int G>
 __host__ __device__ constexpr int volume_nsk_smem() {
   using S = Shape<D, NP>;
-  return G * D * (D + 1) * S::NPE + G * S::NF * (D + 1) * S::NFN + tab_smem<D, NP>();
+  return ((G * D * (D + 1) * S::NPE + G * S::NF * (D + 1) * S::NFN + 1) & ~1) + tab_orig<D, NP>();
 }
 
 // weak-form volume integral and surface lifting of the original NSK equations (no sources),
@@ -200,14 +277,15 @@ __device__ __forceinline__ void volume_group(const NskParams& p, double* __restr
   constexpr int NPE = S::NPE, NFN = S::NFN, NF = S::NF, NQ = S::NQ, NV = D + 1;
   double* sf = sm;                       // [G][D][NV][NPE]
   double* sfs = sm + G * D * NV * NPE;   // [G][NF][NV][NFN]
-  double* tb = sfs + G * NF * NV * NFN;
+  double* tb = sm + ((G * D * NV * NPE + G * NF * NV * NFN + 1) & ~1);
+  constexpr bool FX = fx_on<double, D, NP>();
   const int le = threadIdx.x / NPE, n = threadIdx.x % NPE;
   const int e = (int)e0 + le;
   const bool valid = le < G && e < p.E;
   const size_t nn = (size_t)p.nne;
   const int g = e * NPE + n;
 
-  stage_tables<double, D, NP>(p.td, tb);
+  tables_orig<D, NP>(p, tb);
   double u[NV], kin[NV];
   if (valid) {
 #pragma unroll
@@ -221,27 +299,38 @@ __device__ __forceinline__ void volume_group(const NskParams& p, double* __restr
     for (int c = 0; c < NQ; ++c) q[c] = Q[c * nn + g];
     const double lap = Q2[g];
     eflag |= rho_flags(u[0]);
-    const double dd = 1.0 / (u[0] * (3.0 - u[0]));
+    const double dd = rcp_nr(u[0] * (3.0 - u[0]));
     const double inv = (3.0 - u[0]) * dd;
     const double pr = pressure_q(p, u[0], u[0] * dd);
-    // the symmetric convective momentum flux, each pair k < a formed once
-    double vel[D], off[D][D];
+    // the momentum flux m_k v_a + p delta_ka - tau_ka - tau^K_ka is symmetric: each pair k <= a formed once
+    double vel[D], kg[D], fl[D][D], div = 0.0, g2 = 0.0;
 #pragma unroll
-    for (int a = 0; a < D; ++a) vel[a] = u[1 + a] * inv;
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-#pragma unroll
-      for (int j = i + 1; j < D; ++j) off[i][j] = u[1 + i] * vel[j];
+    for (int a = 0; a < D; ++a) {
+      vel[a] = u[1 + a] * inv;
+      kg[a] = p.kappa * q[a * (D + 1) + D];
+      div += q[a * (D + 1) + a];
+      g2 = fma(q[a * (D + 1) + D], q[a * (D + 1) + D], g2);
+    }
+    const double base = fma(-p.kappa, fma(u[0], lap, 0.5 * g2), pr);
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      double* f = sf + ((le * D + k) * NV) * NPE + n;
-      f[0] = u[1 + k];
-      double fv[D];
-      visc_kort<D>(p, k, u[0], q, lap, fv);
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const double fc = (a == k) ? fma(u[1 + k], vel[k], pr) : (k < a ? off[k][a] : off[a][k]);
-        f[(1 + a) * NPE] = fc - fv[a];
+      for (int a = k; a < D; ++a) {
+        double tau = q[k * (D + 1) + a] + q[a * (D + 1) + k];
+        if (a == k) tau = fma(-2.0 / 3.0, div, tau);
+        const double c = a == k ? fma(u[1 + k], vel[k], base) : u[1 + k] * vel[a];
+        fl[k][a] = fl[a][k] = fma(-p.mu, tau, fma(kg[a], q[k * (D + 1) + D], c));
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const double f = v == 0 ? u[1 + k] : fl[k][v == 0 ? 0 : v - 1];
+        if constexpr (FX)
+          sf[fx_pos<NP>(((le * D + k) * NV + v) * NFN + face_node<D, NP>(n, k), coord<NP>(n, k))] = f;
+        else
+          sf[((le * D + k) * NV + v) * NPE + n] = f;
       }
     }
     const ElemIdx ex = elem_idx<D>(p, e);
@@ -252,7 +341,25 @@ __device__ __forceinline__ void volume_group(const NskParams& p, double* __restr
     }
   }
   __syncthreads();
-  if (valid) {
+  if constexpr (FX) {
+    volume_lines_fx<D, NP, G, NV>(p, tb, sf, sfs, (int)e0);
+    __syncthreads();
+    if (valid) {
+      double res[NV];
+      volume_sums_fx<D, NP, NV>(sf, sfs, le, n, res);
+      const double Bdt = B * dt;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        if (mode == NSK_MODE_RHS) {
+          Rout[v * nn + g] = res[v];
+        } else {
+          const double kv = fma(A, kin[v], res[v]);
+          K[v * nn + g] = kv;
+          U[v * nn + g] = fma(Bdt, kv, u[v]);
+        }
+      }
+    }
+  } else if (valid) {
     double res[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) res[v] = 0.0;
@@ -298,13 +405,22 @@ __global__ void __launch_bounds__(256) k_prolong_nsk(const NskParams p, const do
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < p.nfe) {
     const int e = idx / S::NFN;
-    prolong_trace<double, D, NP, D + 1>(p, U + (size_t)e * S::NPE, (size_t)p.nne, Utr, e, blockIdx.y,
-                                        idx % S::NFN);
+    if constexpr (fx_on<double, D, NP>())
+      prolong_line<D, NP, D + 1>(p, U + (size_t)e * S::NPE, (size_t)p.nne, Utr, e, blockIdx.y, idx % S::NFN);
+    else
+      prolong_trace<double, D, NP, D + 1>(p, U + (size_t)e * S::NPE, (size_t)p.nne, Utr, e, blockIdx.y,
+                                          idx % S::NFN);
   }
 }
 
+// resident warps of the kernels whose contractions are in integers
 template <int D, int NP, int G>
-__global__ void __launch_bounds__(G * Shape<D, NP>::NPE)
+__host__ __device__ constexpr int orig_min_blocks(int warps) {
+  return fx_on<double, D, NP>() ? blocks_in_warps<G * Shape<D, NP>::NPE>(warps) : 1;
+}
+
+template <int D, int NP, int G>
+__global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP, G>(32)))
     k_lift_nsk(const NskParams p, const double* __restrict__ U, const double* __restrict__ Utr,
                double* __restrict__ Q, double* __restrict__ Gtr, int* __restrict__ err) {
   __shared__ __align__(16) double sm[lift_smem<double, D, NP, G>()];
@@ -314,11 +430,11 @@ __global__ void __launch_bounds__(G * Shape<D, NP>::NPE)
 }
 
 template <int D, int NP, int G>
-__global__ void __launch_bounds__(G * Shape<D, NP>::NPE)
+__global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP, G>(24)))
     k_lift2_nsk(const NskParams p, const double* __restrict__ U, const double* __restrict__ Utr,
                 const double* __restrict__ Q, const double* __restrict__ Gtr, double* __restrict__ Q2,
                 double* __restrict__ FVtr) {
-  __shared__ double sm[lift2_work<D, NP, G>() + tab_smem<D, NP>()];
+  __shared__ __align__(16) double sm[((lift2_work<D, NP, G>() + 1) & ~1) + tab_orig<D, NP>()];
   lift2_group<D, NP, G>(p, U, Utr, Q, Gtr, Q2, FVtr, (long long)blockIdx.x * G, sm);
 }
 
@@ -334,12 +450,12 @@ __global__ void __launch_bounds__(256) k_face_nsk(const NskParams p, const doubl
 }
 
 template <int D, int NP, int G>
-__global__ void __launch_bounds__(G * Shape<D, NP>::NPE)
+__global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP, G>(32)))
     k_volume_nsk(const NskParams p, double* __restrict__ U, const double* __restrict__ Q,
                  const double* __restrict__ Q2, const double* __restrict__ Fstar, double* __restrict__ K,
                  double* __restrict__ Rout, const int mode, const double A, const double B,
                  const double* __restrict__ dtp, const double dtv, int* __restrict__ err) {
-  __shared__ double sm[volume_nsk_smem<D, NP, G>()];
+  __shared__ __align__(16) double sm[volume_nsk_smem<D, NP, G>()];
   const double dt = dtp ? *dtp : dtv;
   int eflag = 0;
   volume_group<D, NP, G>(p, U, Q, Q2, Fstar, K, Rout, mode, A, B, dt, (long long)blockIdx.x * G, sm, eflag);
@@ -410,7 +526,7 @@ int launch_stage_g(const NskParams& p, const NskBuffers& b, const NskLaunch& l, 
   using S = Shape<D, NP>;
   int nl = 0;
   if (l.ev) cudaEventRecord(l.ev[0], s);
-  k_prolong_nsk<D, NP><<<dim3(grid_for(p.nfe, 256), S::NF), 256, 0, s>>>(p, (const double*)b.U, (double*)b.Utr);
+  k_prolong_nsk<D, NP><<<dim3(grid_for(p.nfe, 256), prolong_grid_y<double, D, NP>()), 256, 0, s>>>(p, (const double*)b.U, (double*)b.Utr);
   ++nl;
   if (l.ev) cudaEventRecord(l.ev[1], s);
   const unsigned eb = (unsigned)((p.E + G - 1) / G);
