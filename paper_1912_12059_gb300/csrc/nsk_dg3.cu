@@ -23,12 +23,10 @@ int nsk_launch_block_d3(const NskParams& p, int np, bool fp32, const NskBuffers&
   return nsk::launch_block_np_r<double, 3>(p, np, b, mode, coef, dt, nsteps, Rout, s);
 }
 
-// a part of a separate-face stage over an element range (FP64, N = 3, 128 or 256 threads)
+// a part of a separate-face stage over an element range (FP64, N = 3; 128-thread blocks, see small_blocks)
 int nsk_launch_stage_part_d3(const NskParams& p, int np, bool fp32, const NskBuffers& b, const NskLaunch& l,
                              cudaStream_t s, int part, long long e0, long long ne) {
-  if (fp32 || np != 4) return NSK_ERR_ARG;
-  constexpr int G128 = nsk::group_for<3, 4>(128), G256 = nsk::group_for<3, 4>(256);
-  if (l.tpb == 128) return nsk::launch_stage_part<double, 3, 4, G128>(p, b, l, s, part, e0, ne);
-  if (l.tpb == 256) return nsk::launch_stage_part<double, 3, 4, G256>(p, b, l, s, part, e0, ne);
-  return NSK_ERR_ARG;
+  if (fp32 || np != 4 || (l.tpb != 128 && l.tpb != 256)) return NSK_ERR_ARG;
+  static_assert(nsk::small_blocks<double, 3, 4>(256), "the whole stage's launches take the same blocks");
+  return nsk::launch_stage_part<double, 3, 4, nsk::group_for<3, 4>(128)>(p, b, l, s, part, e0, ne);
 }
