@@ -466,17 +466,20 @@ __global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP,
 template <int D>
 __global__ void __launch_bounds__(256) k_dt_nsk(const NskParams p, const long long nn, const double* __restrict__ U,
                                                 unsigned long long* __restrict__ lam, int* __restrict__ err) {
-  double m = 0.0, rmax = 0.0;
+  double m = 0.0, rmax = 0.0, ih = 0.0;  // ih = sum_k 1 / h_k
+#pragma unroll
+  for (int k = 0; k < D; ++k) ih += 0.5 * p.rh[k];
   int eflag = 0;
   for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < nn; g += (long long)gridDim.x * blockDim.x) {
     const double rho = U[g];
     eflag |= rho_flags(rho);
-    const double q = 1.0 / (3.0 - rho);
+    // one integer reciprocal d = 1/(rho (3 - rho)) for 1/rho and 1/(3 - rho)
+    const double r3 = 3.0 - rho, d = rcp_nr(rho * r3), q = rho * d;
     const double dp = fma(p.t24 * q, q, -6.0 * rho);
-    const double a = sqrt(dp > 0.0 ? dp : 0.0);
-    double s = 0.0;
+    double mh = 0.0;  // sum_k |m_k| / h_k
 #pragma unroll
-    for (int k = 0; k < D; ++k) s += (fabs(U[(1 + k) * nn + g] / rho) + a) * (0.5 * p.rh[k]);
+    for (int k = 0; k < D; ++k) mh = fma(fabs(U[(1 + k) * nn + g]), 0.5 * p.rh[k], mh);
+    const double s = fma(r3 * d, mh, sqrt_nr(dp > 0.0 ? dp : 0.0) * ih);
     m = s > m ? s : m;
     rmax = rho > rmax ? rho : rmax;
   }
