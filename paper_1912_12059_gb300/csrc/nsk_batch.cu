@@ -480,57 +480,39 @@ int join_aux(nsk_batch* bt) {
 }
 cudaStream_t inst_stream(const nsk_batch* bt, int i) { return bt->naux < 2 ? bt->stream : bt->aux[i % bt->naux]; }
 
-// instance schedule: every instance's own stage kernels, instance i on stream i mod naux; with
-// stamps (the last stage of a step whose latencies are measured) each instance's completion
-// is stamped right after its last kernel
+// instance schedule: one stage of instance i by its own stage kernels, on stream i mod naux.
 // fused 5: each instance's own schedule (its tpb and fused_face; the lean and single-block schedules
 // run as the separate face pass there)
 int inst_fused(const nsk_ctx* c) { return (c->fused_face == 1 || c->fused_face == 4) ? c->fused_face : 0; }
-int launch_instances(nsk_batch* bt, int mode, double A, double B, int tpb, int fused, int traces,
-                     bool stamps = false) {
-  for (int i = 0; i < bt->n; ++i) {
-    nsk_ctx* c = bt->inst[i];
-    const int fi = fused == 5 ? inst_fused(c) : fused;
-    const int tr = fi == 1 ? 0 : traces;  // the fused volume phase prolongs every stage
-    NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, fused == 5 ? c->tpb : tpb, fi};
-    l.traces_ready = tr & 1;
-    l.utr_next = (tr & 2) ? c->b.Utr : nullptr;  // separate face schedule: written in place
-    const int r = nsk_launch_stage_d3(c->p, c->np, c->precision == NSK_FP32_MIXED, c->b, l, inst_stream(bt, i));
-    if (r < 0) return r;
-    bt->launches += r;
-    if (stamps) {
-      const int st = launch_stamp(bt, bt->d_stamp + 1 + i, 1, inst_stream(bt, i));
-      if (st) return st;
-    }
-  }
-  return NSK_OK;
+int launch_instance(nsk_batch* bt, int i, int mode, double A, double B, int tpb, int fused, int traces) {
+  nsk_ctx* c = bt->inst[i];
+  const int fi = fused == 5 ? inst_fused(c) : fused;
+  const int tr = fi == 1 ? 0 : traces;  // the fused volume phase prolongs every stage
+  NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, fused == 5 ? c->tpb : tpb, fi};
+  l.traces_ready = tr & 1;
+  l.utr_next = (tr & 2) ? c->b.Utr : nullptr;  // separate face schedule: written in place
+  const int r = nsk_launch_stage_d3(c->p, c->np, c->precision == NSK_FP32_MIXED, c->b, l, inst_stream(bt, i));
+  if (r > 0) bt->launches += r;
+  return r;
 }
 
-// the lean stage on every instance (instance schedule, fused_face 2): a step prolongs once into
-// each instance's trace buffer (stage 0), then its stages alternate between that buffer and the
-// instance's spare one (the lean volume kernel writes the next stage's traces while its
-// neighbours still read the current ones); the last stage of a step writes none. stage < 0: a
-// residual (prolongation, no traces written).
-int launch_instances_lean(nsk_batch* bt, int mode, double A, double B, int tpb, int stage, bool stamps) {
-  for (int i = 0; i < bt->n; ++i) {
-    nsk_ctx* c = bt->inst[i];
-    NskBuffers b = c->b;
-    void* bufs[2] = {c->b.Utr, c->utr_alt};
-    NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, tpb, 2};
-    if (stage >= 0) {
-      b.Utr = bufs[stage & 1];
-      l.traces_ready = stage > 0;
-      l.utr_next = stage < 4 ? bufs[(stage + 1) & 1] : nullptr;
-    }
-    const int r = nsk_launch_stage_d3(c->p, c->np, c->precision == NSK_FP32_MIXED, b, l, inst_stream(bt, i));
-    if (r < 0) return r;
-    bt->launches += r;
-    if (stamps) {
-      const int st = launch_stamp(bt, bt->d_stamp + 1 + i, 1, inst_stream(bt, i));
-      if (st) return st;
-    }
+// the lean stage (fused_face 2): a step prolongs once into the instance's trace buffer (stage 0), then
+// its stages alternate between that buffer and the instance's spare one (the lean volume kernel writes
+// the next stage's traces while its neighbours still read the current ones); the last stage of a step
+// writes none. stage < 0: a residual (prolongation, no traces written).
+int launch_instance_lean(nsk_batch* bt, int i, int mode, double A, double B, int tpb, int stage) {
+  nsk_ctx* c = bt->inst[i];
+  NskBuffers b = c->b;
+  void* bufs[2] = {c->b.Utr, c->utr_alt};
+  NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, tpb, 2};
+  if (stage >= 0) {
+    b.Utr = bufs[stage & 1];
+    l.traces_ready = stage > 0;
+    l.utr_next = stage < 4 ? bufs[(stage + 1) & 1] : nullptr;
   }
-  return NSK_OK;
+  const int r = nsk_launch_stage_d3(c->p, c->np, c->precision == NSK_FP32_MIXED, b, l, inst_stream(bt, i));
+  if (r > 0) bt->launches += r;
+  return r;
 }
 
 // the instances' schedules as one number (tpb and effective fused_face of each, in order)
@@ -557,12 +539,11 @@ int launch_batch(nsk_batch* bt, int mode, double A, double B, int tpb, int fused
   if (persistent == 2) {  // the instance schedule, forked onto the auxiliary streams
     int r = fork_aux(bt);
     if (r) return r;
-    if (fused == 2)
-      r = launch_instances_lean(bt, mode, A, B, tpb, stage, stamps);
-    else
-      r = launch_instances(bt, mode, A, B, tpb, fused, fused == 1 ? 0 : traces, stamps);
+    for (int i = 0; i < bt->n && r >= 0; ++i)
+      r = fused == 2 ? launch_instance_lean(bt, i, mode, A, B, tpb, stage)
+                     : launch_instance(bt, i, mode, A, B, tpb, fused, fused == 1 ? 0 : traces);
     const int j = join_aux(bt);
-    return r ? r : j;
+    return r < 0 ? r : j;
   }
   if (fused == 1) traces = 0;  // the fused volume phase reads the traces: they are prolonged every stage
   const int r = persistent ? launch_persistent(bt, mode, A, B, tpb, fused, traces)
@@ -578,6 +559,27 @@ int launch_step(nsk_batch* bt, int dtmode, double cfl, bool stamps) {
     const int st = launch_stamp(bt, bt->d_stamp, 1);
     if (st) return st;
   }
+  if (bt->persistent == 2) {
+    // instance schedule: the instances do not depend on one another, so each runs its whole step (dt and
+    // the five stages) on its stream and the streams join once, at the end of the step: no stage waits for
+    // the slowest instance, and a small instance's arrays stay in the L2 from stage to stage
+    int r = fork_aux(bt);
+    if (r) return r;
+    for (int i = 0; i < bt->n && r >= 0; ++i) {
+      nsk_ctx* c = bt->inst[i];
+      if (dtmode) {
+        r = nsk_launch_dt(c->p, c->dim, c->np, c->precision == NSK_FP32_MIXED, c->b, cfl, inst_stream(bt, i));
+        if (r > 0) bt->launches += r;
+      }
+      const int tr = bt->fused == 1 ? 0 : step_traces(bt->fused);
+      for (int s = 0; s < 5 && r >= 0; ++s)
+        r = bt->fused == 2 ? launch_instance_lean(bt, i, NSK_MODE_LSRK, kA[s], kB[s], bt->tpb, s)
+                           : launch_instance(bt, i, NSK_MODE_LSRK, kA[s], kB[s], bt->tpb, bt->fused, tr);
+      if (stamps && r >= 0) r = launch_stamp(bt, bt->d_stamp + 1 + i, 1, inst_stream(bt, i));
+    }
+    const int j = join_aux(bt);
+    return r < 0 ? r : j;
+  }
   if (dtmode)
     for (nsk_ctx* c : bt->inst) {
       const int r = nsk_launch_dt(c->p, c->dim, c->np, c->precision == NSK_FP32_MIXED, c->b, cfl, bt->stream);
@@ -586,7 +588,7 @@ int launch_step(nsk_batch* bt, int dtmode, double cfl, bool stamps) {
     }
   for (int s = 0; s < 5; ++s) {
     const int r = launch_batch(bt, NSK_MODE_LSRK, kA[s], kB[s], bt->tpb, bt->fused, bt->persistent,
-                               step_traces(bt->fused), stamps && s == 4, s);
+                               step_traces(bt->fused), stamps && s == 4);
     if (r) return r;
   }
   return NSK_OK;
