@@ -14,6 +14,7 @@
 // device: the host reads one number per Arnoldi step, one step behind the GPU, and the triangular
 // system once per GMRES cycle, which it solves; a residual evaluation is one stage launch of the
 // context's pipeline in residual mode on the iterate.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -185,14 +186,16 @@ __global__ void __launch_bounds__(256) k_gs_update(const long long n, const int 
 constexpr int kMaxBlock = 64;  // largest block (nvar npe) the shared-memory inversion takes (2D, N = 3)
 
 // W = U with local unknown (v, node) of every element of colour c raised by
-// eps_e = sqrt(2^-52) (1 + |U|)
-__global__ void __launch_bounds__(256) k_fd_perturb(const long long E, const int npe, const long long nn,
+// eps_e = sqrt(2^-52) (1 + |U|); n values
+__global__ void __launch_bounds__(256) k_fd_perturb(const long long n, const int npe, const long long nn,
                                                     const int* __restrict__ colour, const int c, const int v,
-                                                    const int node, double* __restrict__ W) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (long long)gridDim.x * blockDim.x) {
-    if (colour[e] != c) continue;
-    const size_t g = (size_t)v * nn + e * npe + node;
-    W[g] += sqrt(ldexp(1.0, -52)) * (1.0 + fabs(W[g]));
+                                                    const int node, const double* __restrict__ U,
+                                                    double* __restrict__ W) {
+  for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (long long)gridDim.x * blockDim.x) {
+    double u = U[g];
+    const long long r = g - v * nn;
+    if (r >= 0 && r < nn && r % npe == node && colour[r / npe] == c) u += sqrt(ldexp(1.0, -52)) * (1.0 + fabs(u));
+    W[g] = u;
   }
 }
 
@@ -283,6 +286,7 @@ __global__ void __launch_bounds__(256) k_block_apply(const long long E, const in
 // remaining steps (every kernel of an Arnoldi step returns at once when it is set).
 struct CycleCtl {
   double c0, beta, tol, res;
+  double eps, gnorm, snorm;  // small systems: the step's forward-difference scale, ||G||, ||S_i||
   int kmax, stop, kdone, pad;
 };
 __global__ void k_cycle_init(CycleCtl* ctl, const double c0, const double beta, const double tol, const int kmax) {
@@ -301,10 +305,8 @@ __global__ void k_cycle_init(CycleCtl* ctl, const double c0, const double beta, 
 // and the new vector's norm h2[k + 1]), the earlier Givens rotations applied to it, the new
 // rotation (cs, sn), and the rotated right-hand side gv (gv[0] = beta at k = 0); then the residual
 // estimate |gv[k + 1]|, and stop once it is within the tolerance or the cycle's steps are used up.
-__global__ void k_arnoldi_update(const int k, const int m, const double* __restrict__ h1,
-                                 const double* __restrict__ h2, double* __restrict__ H, double* __restrict__ cs,
-                                 double* __restrict__ sn, double* __restrict__ gv, CycleCtl* __restrict__ ctl) {
-  if (threadIdx.x != 0 || blockIdx.x != 0 || ctl->stop) return;
+__device__ void arnoldi_update(const int k, const int m, const double* h1, const double* h2, double* H, double* cs,
+                               double* sn, double* gv, CycleCtl* ctl) {
   if (k == 0) gv[0] = ctl->beta;
   for (int j = 0; j <= k; ++j) H[(size_t)j * m + k] = h1[j] + h2[j];
   H[(size_t)(k + 1) * m + k] = h2[k + 1];
@@ -325,6 +327,265 @@ __global__ void k_arnoldi_update(const int k, const int m, const double* __restr
   ctl->res = res;
   ctl->kdone = k + 1;
   if (res <= ctl->tol || k + 1 >= ctl->kmax) ctl->stop = 1;
+}
+__global__ void k_arnoldi_update(const int k, const int m, const double* __restrict__ h1,
+                                 const double* __restrict__ h2, double* __restrict__ H, double* __restrict__ cs,
+                                 double* __restrict__ sn, double* __restrict__ gv, CycleCtl* __restrict__ ctl) {
+  if (threadIdx.x != 0 || blockIdx.x != 0 || ctl->stop) return;
+  arnoldi_update(k, m, h1, h2, H, cs, sn, gv, ctl);
+}
+
+// ---- small systems: the vector algebra of an Arnoldi step in two kernels ------------------------
+// On a mesh of a few thousand values every kernel lasts as long as its launch and its latency, and an
+// Arnoldi step was ten (with the preconditioner thirteen) of them around the residual evaluation's four.
+// Here one kernel does everything before the evaluation (preconditioner, forward-difference scale,
+// perturbed state) and one everything after it (difference, both Gram-Schmidt passes, Hessenberg column
+// and rotations); the step index is read from the control block, so one captured graph of kChunk steps
+// serves every chunk of every cycle. Both are one cluster of 8 blocks, each owning an eighth of the vector,
+// that add their partial sums through distributed shared memory: on a single SM the 4 (k + 1) n FP64
+// multiply-adds of the two passes took 22 us at n = 768, k = 30.
+constexpr int kCl = 8, kClThreads = 256;
+constexpr int kSmallN = 4096;
+constexpr long long kSmallBlocks = 65536;  // largest n (nvar npe) of the preconditioner's blocks
+constexpr int kSmallThreads = 1024;
+
+// sums of NS values over the block, valid in every thread (a fixed order)
+template <int NS>
+__device__ __forceinline__ void block_sums(double (&v)[NS], double (*red)[kSmallThreads / 32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    const double t = warp_sum(v[q]);
+    if (lane == 0) red[q][warp] = t;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NS; ++q) v[q] = warp_sum(red[q][lane]);
+}
+
+// row t of the block preconditioner times x: t = e nloc + i, and where local unknown i of element e lies
+struct BlockRows {
+  int npe, nloc;
+  long long nn;
+  const double* Minv;
+  __device__ __forceinline__ size_t at(int t) const {
+    const int e = t / nloc, i = t % nloc;
+    return (size_t)(i / npe) * nn + e * npe + i % npe;
+  }
+  __device__ __forceinline__ double row(int t, const double* x) const {
+    const int e = t / nloc;
+    const double* r = Minv + (size_t)t * nloc;
+    double s = 0.0;
+    for (int v = 0, k = 0; k < nloc; ++v)
+      for (int q = 0; q < npe; ++q, ++k) s = fma(r[k], x[(size_t)v * nn + e * npe + q], s);
+    return s;
+  }
+};
+
+// Newton residual G = X - dtg RX - S, ||G||, ||X||, ||S||, V_0 = -G / ||G|| and the control block of the
+// first GMRES cycle
+__global__ void __launch_bounds__(kSmallThreads) k_small_newton(const int n, const double dtg, const double* X,
+                                                                const double* RX, const double* S, double* V0,
+                                                                const double krylov_tol, const int kmax,
+                                                                CycleCtl* ctl) {
+  __shared__ double red[3][kSmallThreads / 32];
+  double g[kSmallN / kSmallThreads], sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int q = 0; q < kSmallN / kSmallThreads; ++q) {
+    const int i = threadIdx.x + q * kSmallThreads;
+    g[q] = 0.0;
+    if (i < n) {
+      const double x = X[i], b = S[i];
+      g[q] = fma(-dtg, RX[i], x) - b;
+      sum[0] = fma(g[q], g[q], sum[0]);
+      sum[1] = fma(x, x, sum[1]);
+      sum[2] = fma(b, b, sum[2]);
+    }
+  }
+  block_sums<3>(sum, red);
+  const double gn = sqrt(sum[0]), inv = gn > 0.0 ? -1.0 / gn : 0.0;
+#pragma unroll
+  for (int q = 0; q < kSmallN / kSmallThreads; ++q) {
+    const int i = threadIdx.x + q * kSmallThreads;
+    if (i < n) V0[i] = inv * g[q];
+  }
+  if (threadIdx.x == 0) {
+    ctl->c0 = sqrt(ldexp(1.0, -52)) * (1.0 + sqrt(sum[1]));
+    ctl->beta = gn;
+    ctl->tol = krylov_tol * gn;
+    ctl->res = gn;
+    ctl->gnorm = gn;
+    ctl->snorm = sqrt(sum[2]);
+    ctl->kmax = kmax;
+    ctl->stop = 0;
+    ctl->kdone = 0;
+  }
+}
+
+// this block's slice [lo, hi) of the n values
+__device__ __forceinline__ void cl_slice(int n, int rank, int& lo, int& hi) {
+  const int m = (n + kCl - 1) / kCl;
+  lo = min(n, rank * m);
+  hi = min(n, lo + m);
+}
+
+// z = M^-1 V_k into Z (z = V_k without the preconditioner), eps = c0 / ||z|| (c0), W = X + eps z
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
+    k_small_pre(const int n, const BlockRows bl, const double* const* __restrict__ V, const double* __restrict__ X,
+                double* __restrict__ Z, double* __restrict__ W, CycleCtl* __restrict__ ctl) {
+  if (ctl->stop) return;  // the same for every block: it is set after the last read of a step
+  __shared__ double red[kClThreads / 32], part;
+  auto cluster = cooperative_groups::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int lo, hi;
+  cl_slice(n, (int)cluster.block_rank(), lo, hi);
+  const double* v = V[ctl->kdone];
+  constexpr int Q = kSmallN / kCl / kClThreads;
+  double z[Q], zz = 0.0;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int t = lo + threadIdx.x + q * kClThreads;
+    z[q] = 0.0;
+    if (t < hi) z[q] = bl.Minv ? bl.row(t, v) : v[t];
+    zz = fma(z[q], z[q], zz);
+  }
+  double eps = ctl->c0;
+  if (bl.Minv) {
+    zz = warp_sum(zz);
+    if (lane == 0) red[warp] = zz;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < kClThreads / 32; ++w) t += red[w];
+      part = t;
+    }
+    cluster.sync();
+    double t = 0.0;
+#pragma unroll
+    for (int r = 0; r < kCl; ++r) t += *cluster.map_shared_rank(&part, r);
+    eps /= sqrt(t);
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int t = lo + threadIdx.x + q * kClThreads;
+    if (t < hi) {
+      const size_t i = bl.Minv ? bl.at(t) : (size_t)t;
+      if (bl.Minv) Z[i] = z[q];
+      W[i] = fma(eps, z[q], X[i]);
+    }
+  }
+  if (cluster.block_rank() == 0 && threadIdx.x == 0) ctl->eps = eps;
+  cluster.sync();  // a block's shared memory is read by the others until here
+}
+
+// V_{k+1} = z - dtg (R(X + eps z) - R(X)) / eps, orthogonalised twice and normalised, then the Hessenberg
+// column and the rotations
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
+    k_small_post(const int n, const int m, const double dtg, double* const* __restrict__ V, const double* Z,
+                 const double* __restrict__ RW, const double* __restrict__ RX, double* __restrict__ H,
+                 double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ gv,
+                 CycleCtl* __restrict__ ctl) {
+  if (ctl->stop) return;
+  __shared__ double w[kSmallN / kCl], part[2][kMaxNv], h[2][kMaxNv];
+  __shared__ const double* vp[kMaxNv];
+  __shared__ double inv;
+  auto cluster = cooperative_groups::this_cluster();
+  const int k = ctl->kdone, nv = k + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int lo, hi;
+  cl_slice(n, (int)cluster.block_rank(), lo, hi);
+  const double b = dtg / ctl->eps;
+  for (int j = threadIdx.x; j < nv; j += kClThreads) vp[j] = V[j] + lo;
+  double* out = V[nv] + lo;
+  const double* z = Z ? Z : V[k];
+  const int ns = hi - lo;
+  for (int i = threadIdx.x; i < ns; i += kClThreads) w[i] = fma(b, RX[lo + i], fma(-b, RW[lo + i], z[lo + i]));
+  __syncthreads();
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int j = warp; j < nv + pass; j += kClThreads / 32) {  // the second pass: w . w last
+      const double* v = j < nv ? vp[j] : w;
+      double t = 0.0;
+#pragma unroll 4
+      for (int i = lane; i < ns; i += 32) t = fma(v[i], w[i], t);
+      t = warp_sum(t);
+      if (lane == 0) part[pass][j] = t;
+    }
+    cluster.sync();
+    for (int j = threadIdx.x; j < nv + pass; j += kClThreads) {
+      double t = 0.0;
+#pragma unroll
+      for (int r = 0; r < kCl; ++r) t += *cluster.map_shared_rank(&part[pass][j], r);
+      h[pass][j] = t;
+    }
+    __syncthreads();
+    if (pass) {  // ||w - sum h_j V_j|| by Pythagoras
+      if (warp == 0) {
+        double t = 0.0;
+        for (int j = lane; j < nv; j += 32) t = fma(h[1][j], h[1][j], t);
+        t = h[1][nv] - warp_sum(t);
+        const double hn = t > 0.0 ? sqrt(t) : 0.0;
+        __syncwarp();
+        if (lane == 0) {
+          h[1][nv] = hn;
+          inv = hn > 0.0 ? 1.0 / hn : 1.0;
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = threadIdx.x; i < ns; i += kClThreads) {
+      double t = w[i];
+#pragma unroll 4
+      for (int j = 0; j < nv; ++j) t = fma(-h[pass][j], vp[j][i], t);
+      if (pass)
+        out[i] = inv * t;
+      else
+        w[i] = t;
+    }
+    __syncthreads();
+  }
+  cluster.sync();  // a block's partial sums are read by the others until here
+  if (cluster.block_rank() == 0 && threadIdx.x == 0) arnoldi_update(k, m, h[0], h[1], H, cs, sn, gv, ctl);
+}
+
+// End of a cycle of kk steps: back substitution on the rotated Hessenberg matrix, D (+)= M^-1 sum_j y_j V_j
+// (first: D is set), and X += D when the Newton update is complete
+__global__ void __launch_bounds__(kSmallThreads) k_small_solve(const int n, const int m, const int kk,
+                                                               const BlockRows bl, double* const* __restrict__ V,
+                                                               const double* __restrict__ H,
+                                                               const double* __restrict__ gv, double* T, double* D,
+                                                               double* X, const int first, const int final) {
+  __shared__ double y[kMaxNv];
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    for (int r = kk - 1; r >= 0; --r) {
+      double t = 0.0;
+      for (int j = r + 1 + lane; j < kk; j += 32) t = fma(H[(size_t)r * m + j], y[j], t);
+      t = warp_sum(t);
+      if (lane == 0) y[r] = (gv[r] - t) / H[(size_t)r * m + r];
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += kSmallThreads) {
+    double t = 0.0;
+#pragma unroll 4
+    for (int j = 0; j < kk; ++j) t = fma(y[j], V[j][i], t);
+    if (bl.Minv) {
+      T[i] = t;
+    } else {
+      const double d = first ? t : D[i] + t;
+      D[i] = d;
+      if (final) X[i] += d;
+    }
+  }
+  if (!bl.Minv) return;
+  __syncthreads();
+  for (int t = threadIdx.x; t < n; t += kSmallThreads) {
+    const size_t i = bl.at(t);
+    const double z = bl.row(t, T), d = first ? z : D[i] + z;
+    D[i] = d;
+    if (final) X[i] += d;
+  }
 }
 
 // ARK4(3)6L[2]SA, implicit part (Kennedy and Carpenter 2003): a_ij for j < i; gamma = 1/4
@@ -540,14 +801,117 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
     k_block_apply<<<eg, 256, 0, im.s>>>(c->E, c->nvar, c->npe, c->nn, Jb, x, z, im.stop);
     ++im.launches;
   };
+  // restart of a GMRES cycle: V_0 and beta from r = -G - (I - dt gamma J) D; false without progress
+  auto restart = [&](double xn, double& beta) {
+    const double dn = im.norm(D);
+    if (!(dn > 0.0)) return false;  // no progress in this cycle
+    const double eps = sqrt(ldexp(1.0, -52)) * (1.0 + xn) / dn;
+    im.lincomb(1.0, X, eps, D, 0.0, nullptr, W);
+    im.rhs(W, RW);
+    // V_0 = -G - D + (dt gamma / eps)(R(X + eps D) - R(X)); -G from X, RX, S
+    im.lincomb(-1.0, X, gdt, RX, 1.0, S, V[0]);
+    im.lincomb(1.0, V[0], -1.0, D, 0.0, nullptr, V[0]);
+    im.lincomb(1.0, V[0], gdt / eps, RW, -gdt / eps, RX, V[0]);
+    beta = im.norm(V[0]);
+    if (!(beta > 0.0)) return false;
+    im.lincomb(1.0 / beta, V[0], 0.0, nullptr, 0.0, nullptr, V[0]);
+    return true;
+  };
+  const bool small = n <= kSmallN && (!block_precond || n * nloc <= kSmallBlocks);
+  const BlockRows blk = {c->npe, nloc, c->nn, block_precond ? Jb : nullptr};
+  cudaGraphExec_t gchunk = nullptr;  // small systems: kChunk Arnoldi steps
+  long long gchunk_launches = 0;
+  auto read_ctl = [&] {
+    if (cudaMemcpyAsync(hctl, ctl, sizeof(CycleCtl), cudaMemcpyDeviceToHost, im.s) != cudaSuccess ||
+        cudaStreamSynchronize(im.s) != cudaSuccess)
+      im.status = NSK_ERR_CUDA;
+    return im.status == NSK_OK;
+  };
+  auto chunk_small = [&] {  // kChunk Arnoldi steps from the control block's state
+    auto steps = [&] {
+      for (int q = 0; q < kChunk; ++q) {
+        k_small_pre<<<kCl, kClThreads, 0, im.s>>>((int)n, blk, dV, X, Z, W, ctl);
+        im.rhs(W, RW);
+        k_small_post<<<kCl, kClThreads, 0, im.s>>>((int)n, m, gdt, dV, Z, RW, RX, Hd, csd, snd, gvd, ctl);
+        im.launches += 2;
+      }
+    };
+    if (graphs && !gchunk) {
+      const long long l0 = im.launches, r0 = im.rhs_evals;
+      cudaGraph_t g = nullptr;
+      bool ok = cudaStreamBeginCapture(im.s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+      if (ok) {
+        steps();
+        ok = cudaStreamEndCapture(im.s, &g) == cudaSuccess && g && im.status == NSK_OK &&
+             cudaGraphInstantiate(&gchunk, g, 0) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+      }
+      gchunk_launches = im.launches - l0;
+      im.launches = l0;
+      im.rhs_evals = r0;
+      if (!ok) {  // no graph: the steps are launched directly
+        cudaGetLastError();
+        gchunk = nullptr;
+        graphs = false;
+      }
+    }
+    if (!graphs) {
+      steps();
+      return;
+    }
+    if (cudaGraphLaunch(gchunk, im.s) != cudaSuccess) im.status = NSK_ERR_CUDA;
+    im.launches += gchunk_launches;
+    im.rhs_evals += kChunk;
+  };
+  // Newton iterations of one stage of a small system
+  auto newton_small = [&](int) {
+    for (int it = 0;; ++it) {
+      im.rhs(X, RX);
+      k_small_newton<<<1, kSmallThreads, 0, im.s>>>((int)n, gdt, X, RX, S, V[0], krylov_tol, std::min(m, max_krylov),
+                                                    ctl);
+      ++im.launches;
+      if (!read_ctl() || hctl->gnorm <= newton_tol * hctl->snorm) break;
+      if (it == 20) {
+        ++st_fail;
+        break;
+      }
+      const double bn = hctl->gnorm, c0 = hctl->c0, xn = c0 / sqrt(ldexp(1.0, -52)) - 1.0;
+      int its = 0;
+      bool first = true;
+      while (im.status == NSK_OK) {
+        const int kmax = std::min(m, max_krylov - its);
+        for (int k0 = 0; k0 < kmax; k0 += kChunk) {
+          chunk_small();
+          if (!read_ctl() || hctl->stop) break;
+        }
+        const int kk = hctl->kdone;
+        if (im.status != NSK_OK || kk == 0) break;
+        its += kk;
+        const bool done = hctl->res <= krylov_tol * bn || its >= max_krylov;
+        k_small_solve<<<1, kSmallThreads, 0, im.s>>>((int)n, m, kk, blk, dV, Hd, gvd, T, D, X, first, done);
+        ++im.launches;
+        first = false;
+        if (done) break;
+        double beta = 0.0;
+        if (!restart(xn, beta)) {
+          im.lincomb(1.0, X, 1.0, D, 0.0, nullptr, X);
+          break;
+        }
+        k_cycle_init<<<1, 32, 0, im.s>>>(ctl, c0, beta, krylov_tol * bn, std::min(m, max_krylov - its));
+        ++im.launches;
+      }
+      ++st_newton;
+      st_krylov += its;
+      if (im.status != NSK_OK) break;
+    }
+  };
   for (int step = 0; step < nsteps && im.status == NSK_OK; ++step) {
     im.rhs(U, Rj[0]);
     im.lincomb(1.0, U, 0.0, nullptr, 0.0, nullptr, X);
     if (block_precond) {  // blocks of I - dt gamma J(U_n), once per step
       for (int col = 0; col < ncol; ++col)
         for (int k = 0; k < nloc; ++k) {
-          im.lincomb(1.0, U, 0.0, nullptr, 0.0, nullptr, W);
-          k_fd_perturb<<<eg, 256, 0, im.s>>>(c->E, c->npe, c->nn, colour, col, k / c->npe, k % c->npe, W);
+          k_fd_perturb<<<im.grid, 256, 0, im.s>>>(n, c->npe, c->nn, colour, col, k / c->npe, k % c->npe, U, W);
           im.rhs(W, RW);
           k_fd_column<<<eg, 256, 0, im.s>>>(c->E, c->nvar, c->npe, c->nn, colour, col, k, U, RW, Rj[0], Jb);
           im.launches += 2;
@@ -560,6 +924,11 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
       im.lincomb(1.0, U, 0.0, nullptr, 0.0, nullptr, S);
       for (int j = 0; j < i; ++j)
         if (kA6[i][j] != 0.0) im.lincomb(1.0, S, dt * kA6[i][j], Rj[j], 0.0, nullptr, S);
+      if (small) {
+        newton_small(i);
+        if (i < 5) im.lincomb(1.0 / gdt, X, -1.0 / gdt, S, 0.0, nullptr, Rj[i]);
+        continue;
+      }
       const double snorm = im.norm(S);
       for (int it = 0;; ++it) {
         im.rhs(X, RX);
@@ -696,18 +1065,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
           if (resk <= krylov_tol * bn || its >= max_krylov) {
             done = true;
           } else {  // restart: r = -G - (I - dt gamma J) D
-            const double dn = im.norm(D);
-            if (!(dn > 0.0)) break;  // no progress in this cycle
-            const double eps = sqrt(ldexp(1.0, -52)) * (1.0 + xn) / dn;
-            im.lincomb(1.0, X, eps, D, 0.0, nullptr, W);
-            im.rhs(W, RW);
-            // V_0 = -G - D + (dt gamma / eps)(R(X + eps D) - R(X)); -G from X, RX, S
-            im.lincomb(-1.0, X, gdt, RX, 1.0, S, V[0]);
-            im.lincomb(1.0, V[0], -1.0, D, 0.0, nullptr, V[0]);
-            im.lincomb(1.0, V[0], gdt / eps, RW, -gdt / eps, RX, V[0]);
-            beta = im.norm(V[0]);
-            if (!(beta > 0.0)) break;
-            im.lincomb(1.0 / beta, V[0], 0.0, nullptr, 0.0, nullptr, V[0]);
+            if (!restart(xn, beta)) break;
           }
         }
         im.lincomb(1.0, X, 1.0, D, 0.0, nullptr, X);
@@ -734,6 +1092,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
   c->launches += im.launches;
   for (cudaGraphExec_t ge : gstep)
     if (ge) cudaGraphExecDestroy(ge);
+  if (gchunk) cudaGraphExecDestroy(gchunk);
   if (hctl) cudaFreeHost(hctl);
   cudaFree(ctl);
   cudaFree(Jb);
