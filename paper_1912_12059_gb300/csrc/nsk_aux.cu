@@ -25,8 +25,8 @@ int launch_dt_t(const NskParams& p, int np, const NskBuffers& b, double cfl, cud
   for (int k = 0; k < D; ++k) npe *= np;
   const long long nn = p.E * npe;
   if (cudaMemsetAsync(b.lam, 0, sizeof(unsigned long long), s) != cudaSuccess) return NSK_ERR_CUDA;
-  nsk::k_dt<R, D><<<reduce_grid(nn), 256, 0, s>>>(p, nn, (const R*)b.U, b.lam, b.err);
-  nsk::k_dt_final<<<1, 1, 0, s>>>(p, D, np - 1, cfl, b.lam, b.dt);
+  launch_pdl(nsk::k_dt<R, D>, reduce_grid(nn), 256, 0, s, p, nn, (const R*)b.U, b.lam, b.err);
+  launch_pdl(nsk::k_dt_final, 1, 1, 0, s, p, D, np - 1, cfl, b.lam, b.dt);
   return cudaGetLastError() == cudaSuccess ? 2 : NSK_ERR_CUDA;
 }
 

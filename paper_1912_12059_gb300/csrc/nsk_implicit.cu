@@ -388,6 +388,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_newton(const int n, con
                                                                 const double* RX, const double* S, double* V0,
                                                                 const double krylov_tol, const int kmax,
                                                                 CycleCtl* ctl) {
+  pdl_begin();
   __shared__ double red[3][kSmallThreads / 32];
   double g[kSmallN / kSmallThreads], sum[3] = {0.0, 0.0, 0.0};
 #pragma unroll
@@ -433,6 +434,7 @@ __device__ __forceinline__ void cl_slice(int n, int rank, int& lo, int& hi) {
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     k_small_pre(const int n, const BlockRows bl, const double* const* __restrict__ V, const double* __restrict__ X,
                 double* __restrict__ Z, double* __restrict__ W, CycleCtl* __restrict__ ctl) {
+  pdl_begin();
   if (ctl->stop) return;  // the same for every block: it is set after the last read of a step
   __shared__ double red[kClThreads / 32], part;
   auto cluster = cooperative_groups::this_cluster();
@@ -485,6 +487,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
                  const double* __restrict__ RW, const double* __restrict__ RX, double* __restrict__ H,
                  double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ gv,
                  CycleCtl* __restrict__ ctl) {
+  pdl_begin();
   if (ctl->stop) return;
   __shared__ double w[kSmallN / kCl], part[2][kMaxNv], h[2][kMaxNv];
   __shared__ const double* vp[kMaxNv];
@@ -554,6 +557,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_solve(const int n, cons
                                                                const double* __restrict__ H,
                                                                const double* __restrict__ gv, double* T, double* D,
                                                                double* X, const int first, const int final) {
+  pdl_begin();
   __shared__ double y[kMaxNv];
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 32) {
@@ -830,9 +834,9 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
   auto chunk_small = [&] {  // kChunk Arnoldi steps from the control block's state
     auto steps = [&] {
       for (int q = 0; q < kChunk; ++q) {
-        k_small_pre<<<kCl, kClThreads, 0, im.s>>>((int)n, blk, dV, X, Z, W, ctl);
+        launch_pdl(k_small_pre, kCl, kClThreads, 0, im.s, (int)n, blk, dV, X, Z, W, ctl);
         im.rhs(W, RW);
-        k_small_post<<<kCl, kClThreads, 0, im.s>>>((int)n, m, gdt, dV, Z, RW, RX, Hd, csd, snd, gvd, ctl);
+        launch_pdl(k_small_post, kCl, kClThreads, 0, im.s, (int)n, m, gdt, dV, Z, RW, RX, Hd, csd, snd, gvd, ctl);
         im.launches += 2;
       }
     };
@@ -867,7 +871,8 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
   auto newton_small = [&](int) {
     for (int it = 0;; ++it) {
       im.rhs(X, RX);
-      k_small_newton<<<1, kSmallThreads, 0, im.s>>>((int)n, gdt, X, RX, S, V[0], krylov_tol, std::min(m, max_krylov),
+      launch_pdl(k_small_newton, 1, kSmallThreads, 0, im.s, (int)n, gdt, X, RX, S, V[0], krylov_tol, std::min(m,
+                 max_krylov),
                                                     ctl);
       ++im.launches;
       if (!read_ctl() || hctl->gnorm <= newton_tol * hctl->snorm) break;
@@ -888,7 +893,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
         if (im.status != NSK_OK || kk == 0) break;
         its += kk;
         const bool done = hctl->res <= krylov_tol * bn || its >= max_krylov;
-        k_small_solve<<<1, kSmallThreads, 0, im.s>>>((int)n, m, kk, blk, dV, Hd, gvd, T, D, X, first, done);
+        launch_pdl(k_small_solve, 1, kSmallThreads, 0, im.s, (int)n, m, kk, blk, dV, Hd, gvd, T, D, X, first, done);
         ++im.launches;
         first = false;
         if (done) break;

@@ -198,6 +198,30 @@ int nsk_launch_diag(const NskParams& p, int dim, int np, bool fp32, const NskBuf
 // precision conversion of nodal arrays (FP32 mode boundary)
 int nsk_launch_convert(const void* src, bool src64, void* dst, bool dst64, long long n, cudaStream_t s);
 
+// Programmatic dependent launch: a kernel launched with launch_pdl may start while its predecessor in the
+// stream drains; it runs pdl_begin before its first global access, which lets the next such kernel start
+// in turn and waits until the predecessor has completed and its writes are visible. Every kernel so launched
+// begins with it, so the order of all memory accesses is that of ordinary launches; the launch latency and
+// the ramp-up of a kernel overlap its predecessor's last blocks (about 2 us per launch boundary).
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);  // errors are read by the callers' cudaGetLastError
+}
+
 // One context (the opaque nsk_ctx of the ABI): mesh, parameters, device buffers.
 // Device buffers of the 1D sub-cell path (nsk_fv.cu)
 struct FvBuffers {

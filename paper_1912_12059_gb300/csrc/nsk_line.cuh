@@ -46,6 +46,7 @@ template <int G>
 __global__ void __launch_bounds__(G * 16, lift_line_min_blocks<G>())
     k_lift_line(const NskParams p, const float* __restrict__ U, const float* __restrict__ Utr,
                 float* __restrict__ Q, float* __restrict__ FVtr, int* __restrict__ err) {
+  pdl_begin();
   using R = float;
   using namespace line;
   extern __shared__ __align__(16) unsigned char line_smem_raw[];
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(G * 16)
                   const float* __restrict__ Fstar, float* __restrict__ K, float* __restrict__ Rout, const int mode,
                   const float A, const float B, const double* __restrict__ dtp, const float dtv,
                   int* __restrict__ err, float* __restrict__ UtrNext) {
+  pdl_begin();
   using R = float;
   using namespace line;
   extern __shared__ __align__(16) unsigned char line_smem_raw[];
@@ -513,27 +515,29 @@ int launch_stage_line(const NskParams& p, const NskBuffers& b, const NskLaunch& 
   int nl = 0;
   if (l.ev) cudaEventRecord(l.ev[0], s);
   if (!l.traces_ready) {
-    k_prolong<float, 3, 4><<<dim3(grid_for(p.nfe, 256), 6), 256, 0, s>>>(p, (const float*)b.U, (float*)b.Utr);
+    launch_pdl(k_prolong<float, 3, 4>, dim3(grid_for(p.nfe, 256), 6), 256, 0, s, p, (const float*)b.U, (float*)b.Utr,
+               0);
     ++nl;
   }
   if (l.ev) cudaEventRecord(l.ev[1], s);
   const unsigned eb = (unsigned)((p.E + G - 1) / G);
   if (l.mode == NSK_MODE_LIFT) {
     constexpr int GN = group_for<3, 4>(256);
-    k_lift<float, 3, 4, GN, false><<<(unsigned)((p.E + GN - 1) / GN), GN * 64, 0, s>>>(
-        p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q, (float*)b.FVtr, b.err);
+    launch_pdl(k_lift<float, 3, 4, GN, false>, (unsigned)((p.E + GN - 1) / GN), GN * 64, 0, s,
+        p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q, (float*)b.FVtr, b.err, 0);
   } else {
-    k_lift_line<G><<<eb, G * 16, smem_lift, s>>>(p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q,
+    launch_pdl(k_lift_line<G>, eb, G * 16, smem_lift, s, p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q,
                                                  (float*)b.FVtr, b.err);
   }
   if (l.ev) cudaEventRecord(l.ev[2], s);
   ++nl;
   if (l.mode != NSK_MODE_LIFT) {
-    k_face<float, 3, 4><<<dim3(grid_for(p.nfe, 256), 3), 256, 0, s>>>(p, (const float*)b.Utr, (const float*)b.FVtr,
-                                                                       (float*)b.Fstar, b.err);
+    launch_pdl(k_face<float, 3, 4>, dim3(grid_for(p.nfe, 256), 3), 256, 0, s, p, (const float*)b.Utr,
+               (const float*)b.FVtr,
+                                                                       (float*)b.Fstar, b.err, 0);
     ++nl;
     if (l.ev) cudaEventRecord(l.ev[3], s);
-    k_volume_line<G><<<eb, G * 16, smem_vol, s>>>(p, (float*)b.U, (const float*)b.Q, (const float*)b.Fstar,
+    launch_pdl(k_volume_line<G>, eb, G * 16, smem_vol, s, p, (float*)b.U, (const float*)b.Q, (const float*)b.Fstar,
                                                   (float*)b.K, (float*)l.Rout, l.mode, (float)l.A, (float)l.B,
                                                   l.dt_dev, (float)l.dt_val, b.err, (float*)l.utr_next);
     if (l.ev) cudaEventRecord(l.ev[4], s);

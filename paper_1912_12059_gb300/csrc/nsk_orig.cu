@@ -401,6 +401,7 @@ __device__ __forceinline__ void volume_group(const NskParams& p, double* __restr
 template <int D, int NP>
 __global__ void __launch_bounds__(256) k_prolong_nsk(const NskParams p, const double* __restrict__ U,
                                                      double* __restrict__ Utr) {
+  pdl_begin();
   using S = Shape<D, NP>;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < p.nfe) {
@@ -423,6 +424,7 @@ template <int D, int NP, int G>
 __global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP, G>(32)))
     k_lift_nsk(const NskParams p, const double* __restrict__ U, const double* __restrict__ Utr,
                double* __restrict__ Q, double* __restrict__ Gtr, int* __restrict__ err) {
+  pdl_begin();
   __shared__ __align__(16) double sm[lift_smem<double, D, NP, G>()];
   int eflag = 0;
   lift_group<double, D, NP, G, 1>(p, U, Utr, Q, Gtr, (long long)blockIdx.x * G, sm, eflag);
@@ -434,6 +436,7 @@ __global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP,
     k_lift2_nsk(const NskParams p, const double* __restrict__ U, const double* __restrict__ Utr,
                 const double* __restrict__ Q, const double* __restrict__ Gtr, double* __restrict__ Q2,
                 double* __restrict__ FVtr) {
+  pdl_begin();
   __shared__ __align__(16) double sm[((lift2_work<D, NP, G>() + 1) & ~1) + tab_orig<D, NP>()];
   lift2_group<D, NP, G>(p, U, Utr, Q, Gtr, Q2, FVtr, (long long)blockIdx.x * G, sm);
 }
@@ -442,6 +445,7 @@ template <int D, int NP>
 __global__ void __launch_bounds__(256) k_face_nsk(const NskParams p, const double* __restrict__ Utr,
                                                   const double* __restrict__ FVtr, double* __restrict__ Fstar,
                                                   int* __restrict__ err) {
+  pdl_begin();
   using S = Shape<D, NP>;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   int eflag = 0;
@@ -455,6 +459,7 @@ __global__ void __launch_bounds__(G * Shape<D, NP>::NPE, (orig_min_blocks<D, NP,
                  const double* __restrict__ Q2, const double* __restrict__ Fstar, double* __restrict__ K,
                  double* __restrict__ Rout, const int mode, const double A, const double B,
                  const double* __restrict__ dtp, const double dtv, int* __restrict__ err) {
+  pdl_begin();
   __shared__ __align__(16) double sm[volume_nsk_smem<D, NP, G>()];
   const double dt = dtp ? *dtp : dtv;
   int eflag = 0;
@@ -529,26 +534,28 @@ int launch_stage_g(const NskParams& p, const NskBuffers& b, const NskLaunch& l, 
   using S = Shape<D, NP>;
   int nl = 0;
   if (l.ev) cudaEventRecord(l.ev[0], s);
-  k_prolong_nsk<D, NP><<<dim3(grid_for(p.nfe, 256), prolong_grid_y<double, D, NP>()), 256, 0, s>>>(p, (const double*)b.U, (double*)b.Utr);
+  launch_pdl(k_prolong_nsk<D, NP>, dim3(grid_for(p.nfe, 256), prolong_grid_y<double, D, NP>()), 256, 0, s, p,
+             (const double*)b.U, (double*)b.Utr);
   ++nl;
   if (l.ev) cudaEventRecord(l.ev[1], s);
   const unsigned eb = (unsigned)((p.E + G - 1) / G);
-  k_lift_nsk<D, NP, G><<<eb, G * S::NPE, 0, s>>>(p, (const double*)b.U, (const double*)b.Utr, (double*)b.Q,
+  launch_pdl(k_lift_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (const double*)b.U, (const double*)b.Utr, (double*)b.Q,
                                                   (double*)b.Gtr, b.err);
   ++nl;
   if (l.mode != NSK_MODE_LIFT) {
-    k_lift2_nsk<D, NP, G><<<eb, G * S::NPE, 0, s>>>(p, (const double*)b.U, (const double*)b.Utr,
+    launch_pdl(k_lift2_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (const double*)b.U, (const double*)b.Utr,
                                                      (const double*)b.Q, (const double*)b.Gtr, (double*)b.Q2,
                                                      (double*)b.FVtr);
     ++nl;
   }
   if (l.ev) cudaEventRecord(l.ev[2], s);
   if (l.mode != NSK_MODE_LIFT) {
-    k_face_nsk<D, NP><<<dim3(grid_for(p.nfe, 256), D), 256, 0, s>>>(p, (const double*)b.Utr, (const double*)b.FVtr,
+    launch_pdl(k_face_nsk<D, NP>, dim3(grid_for(p.nfe, 256), D), 256, 0, s, p, (const double*)b.Utr,
+               (const double*)b.FVtr,
                                                                      (double*)b.Fstar, b.err);
     ++nl;
     if (l.ev) cudaEventRecord(l.ev[3], s);
-    k_volume_nsk<D, NP, G><<<eb, G * S::NPE, 0, s>>>(p, (double*)b.U, (const double*)b.Q, (const double*)b.Q2,
+    launch_pdl(k_volume_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (double*)b.U, (const double*)b.Q, (const double*)b.Q2,
                                                       (const double*)b.Fstar, (double*)b.K, (double*)l.Rout, l.mode,
                                                       l.A, l.B, l.dt_dev, l.dt_val, b.err);
     ++nl;

@@ -488,6 +488,7 @@ struct ChunkWalk {
 // be fewer, a multiple of 16), so that a batch of few row tiles still fills the SMs; a column's sum does
 // not depend on the split.
 __global__ void __launch_bounds__(kRbThreads, 1) k_gemm_tc_rb(const GemmArgs a) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem[];
   const int K = a.K, n0 = blockIdx.y * a.nslice, N = a.nslice ? min(a.nslice, a.N - n0) : a.N;
   unsigned char* sB = smem;
@@ -623,6 +624,7 @@ __device__ __forceinline__ void red_add_v4(float* p, float4 v) {
 }
 
 __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const WgradArgs a) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) unsigned long long mbar;
   __shared__ uint32_t tmem_slot;
@@ -703,7 +705,7 @@ inline int launch_wgrad(WgradArgs& a, cudaStream_t s) {
   a.tile0[0] = 0;
   for (int l = 0; l < 3; ++l) a.tile0[l + 1] = a.tile0[l] + (a.job[l].M + kBM - 1) / kBM;
   a.ks = a.batch < kWgK ? a.batch : kWgK;
-  k_wgrad<<<dim3((unsigned)a.tile0[3], (unsigned)((a.batch + a.ks - 1) / a.ks)), kWgThreads, kWgSmem, s>>>(a);
+  launch_pdl(k_wgrad, dim3((unsigned)a.tile0[3], (unsigned)((a.batch + a.ks - 1) / a.ks)), kWgThreads, kWgSmem, s, a);
   return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
@@ -1485,12 +1487,12 @@ inline int launch_gemm(const GemmArgs& a, cudaStream_t s) {
     int smem = rb_b_bytes(b.nslice, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
     const int gx = (int)persistent_grid(ntiles, sms / ny > 0 ? sms / ny : 1);
-    k_gemm_tc_rb<<<dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s>>>(b);
+    launch_pdl(k_gemm_tc_rb, dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s, b);
   } else if (resident) {
     int smem = rb_b_bytes(a.N, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
     if (smem > kRbSmemMax) return NSK_ERR_ARG;
-    k_gemm_tc_rb<<<persistent_grid(ntiles, sms), kRbThreads, smem, s>>>(a);
+    launch_pdl(k_gemm_tc_rb, persistent_grid(ntiles, sms), kRbThreads, smem, s, a);
   } else {
     dim3 grid((unsigned)((a.M + kBM - 1) / kBM), (unsigned)((a.K + a.k_split - 1) / a.k_split));
     k_gemm_tc<<<grid, kThreads, kSmemBytes, s>>>(a);
