@@ -489,15 +489,21 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
                  CycleCtl* __restrict__ ctl) {
   pdl_begin();
   if (ctl->stop) return;
-  __shared__ double w[kSmallN / kCl], part[2][kMaxNv], h[2][kMaxNv];
+  __shared__ double w[kSmallN / kCl], part[2][kMaxNv], h[2][kMaxNv], rc[kMaxNv], rs[kMaxNv];
   __shared__ const double* vp[kMaxNv];
   __shared__ double inv;
   auto cluster = cooperative_groups::this_cluster();
   const int k = ctl->kdone, nv = k + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int lo, hi;
   cl_slice(n, (int)cluster.block_rank(), lo, hi);
-  const double b = dtg / ctl->eps;
-  for (int j = threadIdx.x; j < nv; j += kClThreads) vp[j] = V[j] + lo;
+  const double b = dtg / ctl->eps, gk = k == 0 ? ctl->beta : gv[k];
+  for (int j = threadIdx.x; j < nv; j += kClThreads) {
+    vp[j] = V[j] + lo;
+    if (j < k) {  // the earlier rotations, for the tail below
+      rc[j] = cs[j];
+      rs[j] = sn[j];
+    }
+  }
   double* out = V[nv] + lo;
   const double* z = Z ? Z : V[k];
   const int ns = hi - lo;
@@ -547,7 +553,31 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     __syncthreads();
   }
   cluster.sync();  // a block's partial sums are read by the others until here
-  if (cluster.block_rank() == 0 && threadIdx.x == 0) arnoldi_update(k, m, h[0], h[1], H, cs, sn, gv, ctl);
+  if (cluster.block_rank() != 0) return;
+  // arnoldi_update with the column and the rotations in shared memory: from global memory each of the k
+  // serial rotations waited for the L2
+  double* col = h[0];
+  for (int j = threadIdx.x; j < nv; j += kClThreads) col[j] += h[1][j];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int j = 0; j < k; ++j) {
+      const double x = col[j], y = col[j + 1];
+      col[j] = rc[j] * x + rs[j] * y;
+      col[j + 1] = -rs[j] * x + rc[j] * y;
+    }
+    const double x = col[k], y = h[1][nv], d = hypot(x, y), c = x / d, s = y / d, gn = -s * gk;
+    col[k] = d;
+    cs[k] = c;
+    sn[k] = s;
+    gv[k + 1] = gn;
+    gv[k] = c * gk;
+    const double res = fabs(gn);
+    ctl->res = res;
+    ctl->kdone = k + 1;
+    if (res <= ctl->tol || k + 1 >= ctl->kmax) ctl->stop = 1;
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j <= nv; j += kClThreads) H[(size_t)j * m + k] = j < nv ? col[j] : 0.0;
 }
 
 // End of a cycle of kk steps: back substitution on the rotated Hessenberg matrix, D (+)= M^-1 sum_j y_j V_j
@@ -558,14 +588,22 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_solve(const int n, cons
                                                                const double* __restrict__ gv, double* T, double* D,
                                                                double* X, const int first, const int final) {
   pdl_begin();
-  __shared__ double y[kMaxNv];
+  constexpr int kHs = 48;  // triangles up to this size are solved from shared memory
+  __shared__ double y[kMaxNv], hs[kHs * kHs];
   const int lane = threadIdx.x & 31;
+  const bool in_smem = kk <= kHs;
+  if (in_smem) {
+    for (int t = threadIdx.x; t < kk * kk; t += kSmallThreads) hs[t] = H[(size_t)(t / kk) * m + t % kk];
+    for (int j = threadIdx.x; j < kk; j += kSmallThreads) y[j] = gv[j];
+    __syncthreads();
+  }
   if (threadIdx.x < 32) {
     for (int r = kk - 1; r >= 0; --r) {
+      const double* row = in_smem ? hs + r * kk : H + (size_t)r * m;
       double t = 0.0;
-      for (int j = r + 1 + lane; j < kk; j += 32) t = fma(H[(size_t)r * m + j], y[j], t);
+      for (int j = r + 1 + lane; j < kk; j += 32) t = fma(row[j], y[j], t);
       t = warp_sum(t);
-      if (lane == 0) y[r] = (gv[r] - t) / H[(size_t)r * m + r];
+      if (lane == 0) y[r] = ((in_smem ? y[r] : gv[r]) - t) / row[r];
       __syncwarp();
     }
   }
