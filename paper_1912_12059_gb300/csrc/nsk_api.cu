@@ -385,8 +385,8 @@ bool block_eligible(const nsk_ctx* c) {
          nsk_block_bytes(c->dim, c->p, c->np, c->precision == NSK_FP32_MIXED) <= (size_t)kBlockSmemMax;
 }
 
-// one launch of the single-block kernel: nsteps LSRK steps at the fixed dt, or (nsteps = 0) one
-// residual into l.Rout; profiled as kernel 4
+// one launch of the single-block kernel: nsteps LSRK steps at the fixed dt, or (Rout set) the residual,
+// nsteps times over, into Rout; profiled as kernel 4
 int launch_block(nsk_ctx* c, int nsteps, double dt, void* Rout) {
   cudaEvent_t* ev = prof_group(c, 16);
   if (ev) cudaEventRecord(ev[4], c->stream);
@@ -396,7 +396,7 @@ int launch_block(nsk_ctx* c, int nsteps, double dt, void* Rout) {
     coef.B[i] = kB[i];
   }
   const int r = nsk_launch_block(c->dim, c->p, c->np, c->precision == NSK_FP32_MIXED, c->b,
-                                 nsteps > 0 ? NSK_MODE_LSRK : NSK_MODE_RHS, coef, dt, nsteps > 0 ? nsteps : 1, Rout,
+                                 Rout ? NSK_MODE_RHS : NSK_MODE_LSRK, coef, dt, nsteps, Rout,
                                  c->stream);
   if (ev) cudaEventRecord(ev[5], c->stream);
   if (r < 0) return r;
@@ -412,7 +412,7 @@ bool line_eligible(const nsk_ctx* c) {
 
 int launch_stage(nsk_ctx* c, NskLaunch l) {
   if (l.fused_face == 3) {  // single-block schedule: a residual in one launch; otherwise the separate face pass
-    if (l.mode == NSK_MODE_RHS && block_eligible(c)) return launch_block(c, 0, 0.0, l.Rout);
+    if (l.mode == NSK_MODE_RHS && block_eligible(c)) return launch_block(c, 1, 0.0, l.Rout);
     l.fused_face = 0;
   }
   // kernels 0..3 = prolong, lift, face, volume
@@ -1168,14 +1168,21 @@ int nsk_autotune(nsk_ctx* c, int* tpb_out, int* fused_out, double* ms_out) {
       // volume kernel (to the spare buffer: U does not change in RHS mode)
       l.traces_ready = 1;
       l.utr_next = c->utr_alt;
+      // (the single-block schedule runs a step's five stages in one launch: a launch per residual, 13.2 us
+      // with 64 1D elements, would lose to separate kernels at 11.8, which overlap their launches and
+      // take 14.8 a stage in a step against its 10.2)
+      const int reps = sched[f] == 3 ? 5 : 3;
       cudaEventRecord(e0, c->stream);
-      for (int r = 0; r < 3 && st == NSK_OK; ++r) st = launch_stage(c, l);
+      if (sched[f] == 3)
+        st = launch_block(c, reps, 0.0, c->rbuf);
+      else
+        for (int r = 0; r < reps && st == NSK_OK; ++r) st = launch_stage(c, l);
       cudaEventRecord(e1, c->stream);
       if (cudaEventSynchronize(e1) != cudaSuccess) st = NSK_ERR_CUDA;
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
-      if (st == NSK_OK && ms / 3.0 < best) {
-        best = ms / 3.0;
+      if (st == NSK_OK && ms / reps < best) {
+        best = ms / reps;
         bt = c->tpb;
         bf = c->fused_face;
       }
