@@ -46,13 +46,13 @@ def compulsory_bytes(d, fp_bytes):
     return 4 * (d + 2) * fp_bytes
 
 
-# DRAM bytes (read + write) per launch of a kernel at 64^3 elements, N = 3, from one ncu capture
-# at 40^3 elements of the same kernel source, scaled by the element count; None once the kernel
+# DRAM bytes (read + write) per launch of a kernel at 64^3 elements, N = 3, from one ncu capture of
+# the same kernel source on a smaller mesh, scaled by the element count; None once the kernel
 # changed after the capture (then no traffic is claimed). FP64: k_volume (separate face pass,
-# 11,671 + 9,600 B per element); FP32: the line schedule's volume kernel, k_volume_line
-# (5.83 + 3.63 KB per element).
-MEASURED_TRAFFIC = {("k_volume", 8, 262144): 5.576e9, ("k_volume", 4, 262144): 2.480e9}
-TRAFFIC_SOURCE = "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch at 40^3 elements, scaled to 64^3"
+# 11,756 + 9,759 B per element at 40^3); FP32: the line schedule's volume kernel, k_volume_line
+# (5.83 + 3.99 KB per element at 48^3).
+MEASURED_TRAFFIC = {("k_volume", 8, 262144): 5.640e9, ("k_volume", 4, 262144): 2.576e9}
+TRAFFIC_SOURCE = "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on a smaller mesh, scaled to 64^3"
 
 
 def alu_peak_tflops(sms, sm_mhz, fp64=True):
@@ -423,7 +423,9 @@ def run_gpu(args, wl, rank, world):
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     max_mhz = clocks["sm_max_mhz"] or float(peaks.get("sm_max_mhz", 2070.0))
     traffic = MEASURED_TRAFFIC.get((name, fp_bytes, s.E))
-    if prec == nsk.NSK_FP64:
+    # 2D/3D FP64 contractions with N >= 2 run on the integer pipe: the counted flops are no longer FP64
+    # issue slots there, and the kernel is held against memory on the bytes it has to move
+    if prec == nsk.NSK_FP64 and (wl.dim < 2 or wl.N < 2):
         peak = alu_peak_tflops(sms, max_mhz, fp64=True)
         achieved = flops_e * s.E / (avg_ms / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
@@ -437,6 +439,9 @@ def run_gpu(args, wl, rank, world):
         roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                 "traffic": traffic, "kernel": name, "peak_source": hbm_src,
                 "algorithmic_per_launch": bytes_e * s.E}
+        if prec == nsk.NSK_FP64:
+            roof["probe_fp64_tflops"] = probe64
+            roof["probe_sm_mhz_median"] = probe_clk
     roof["traffic_source"] = TRAFFIC_SOURCE if traffic is not None else None
     # the whole step against HBM on the compulsory bytes (U and K read and written once per stage)
     step_bytes = compulsory_bytes(wl.dim, fp_bytes) * total_nodes * 5 * args.steps

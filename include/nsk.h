@@ -247,9 +247,8 @@ int nsk_step_host(nsk_ctx* ctx, const double* U_in, double* U_out, double dt, in
  * iterations, Krylov iterations, residual evaluations, stages stopped at the iteration limit,
  * summed over the call. FP64 contexts with the explicit c equation and without the sub-cell
  * path only (NSK_ERR_ARG otherwise). Allocates 12 + krylov_dim state-sized FP64 buffers for the
- * call and frees them before returning. The GMRES control runs on the host: each Krylov iteration
- * reads its projection coefficients and new norm back once (one stream synchronisation), and
- * each Newton iteration its norms. */
+ * call and frees them before returning. The GMRES control runs on the host: it reads a control block
+ * back every four Krylov iterations and once per Newton iteration (one stream synchronisation each). */
 int nsk_step_esdirk(nsk_ctx* ctx, double dt, int nsteps, double newton_tol, double krylov_tol, int krylov_dim,
                     int max_krylov, int block_precond, long long stats[4]);
 
@@ -311,9 +310,11 @@ int nsk_measure_fma_rate(int precision, int iters, double* tflops, double* ms, v
  *     (16 threads per element, each owning a line of 4 nodes: 16-byte loads
  *     and stores, contractions along the line in registers); elsewhere the
  *     separate face pass runs.
- * Default: tpb 256, separate face pass. Every expression that could be
+ * Default: tpb 256, separate face pass. (FP64 elements in 2D and 3D with
+ * N >= 3 always run 128-thread blocks: faster at every size measured.) Every expression that could be
  * contracted into a fused multiply-add in more than one way is written as an
- * explicit fma, and every schedule evaluates each value with the same code,
+ * explicit fma (and the FP64 line contractions in 2D and 3D with N >= 2 are exact integer sums,
+ * rounded once), and every schedule evaluates each value with the same code,
  * so results are bit-identical under every schedule. NSK_ERR_ARG for other
  * values. */
 int nsk_set_schedule(nsk_ctx* ctx, int tpb, int fused_face);
@@ -349,9 +350,9 @@ int nsk_batch_create(nsk_batch** out, int n, nsk_ctx* const* instances);
  * ([step][instance], ms): the time from the start of the step to the moment
  * that instance's new state is complete in device memory, from the GPU's
  * global timer read by one-thread kernels at the start of the step and right
- * after the launch that finishes the instance (the instance schedule runs
- * instance i on stream i mod 4 of four streams forked from the batch's stream
- * and joined back after every stage, and finishes the instances of one stream
+ * after the launch that finishes the instance (the instance schedule runs the
+ * whole step of instance i on stream i mod 4 of four streams forked from the batch's stream
+ * and joined back at the end of the step, and finishes the instances of one stream
  * one after another; the single-launch schedules finish all of them with their
  * last launch). The stamps add n + 1 tiny launches
  * to a measured step (a separately captured graph) and a device-to-device

@@ -18,10 +18,9 @@
 // result's error is smaller than that of the FP64 sums it replaces, and it does not depend on the
 // order of the terms or on the thread that forms it.
 //
-// Measured (64^3 elements, N = 3, 256 threads, per stage): lifting 3.77 -> 1.87 ms, volume 5.15 -> 3.02
-// ms, prolongation 1.35 -> 0.60 ms. Bound now: the lifting by integer issue (ALU pipe 52 %, FP64 48 %,
-// issue slots 51 % busy at 32 resident warps), the volume kernel by latency at 16 resident warps
-// (FP64 53 %, ALU 36 %).
+// Measured (64^3 elements, N = 3, ms a stage, FP64 sums before): lifting 3.77 -> 1.43, volume 5.15 ->
+// 1.73, prolongation 1.35 -> 0.56. Bound now: the lifting by integer issue (ALU pipe 68 %, issue slots
+// 62 %, FP64 32 %), the volume kernel by both pipes (FP64 66 %, ALU 64 %) at 3.1 TB/s of DRAM traffic.
 //
 // Bounds: |h| <= 2^30, pair sums and differences in [-2^31, 2^31 - 1] and their low limbs below 2^29 in
 // magnitude, row sums of |matrix h| <= 2^30, at most 4 terms a product sum: |sum h h| <= 2^61,

@@ -11,9 +11,10 @@
 // the later stages use R_i = (X_i - S_i) / (dt gamma). The vector algebra runs in the kernels
 // below (dot products in a fixed order: deterministic), with the scales, the projection
 // coefficients, the Hessenberg matrix, the Givens rotations and the residual estimate kept on the
-// device: the host reads one number per Arnoldi step, one step behind the GPU, and the triangular
-// system once per GMRES cycle, which it solves; a residual evaluation is one stage launch of the
-// context's pipeline in residual mode on the iterate.
+// device: the host reads one control block per kChunk Arnoldi steps and, for large systems, the triangular
+// system once per GMRES cycle, which it solves; systems of up to kSmallN unknowns run two cluster kernels
+// around each residual evaluation and solve the triangle on the device. A residual evaluation is one
+// stage launch of the context's pipeline in residual mode on the iterate.
 #include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
@@ -909,9 +910,8 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
   auto newton_small = [&](int) {
     for (int it = 0;; ++it) {
       im.rhs(X, RX);
-      launch_pdl(k_small_newton, 1, kSmallThreads, 0, im.s, (int)n, gdt, X, RX, S, V[0], krylov_tol, std::min(m,
-                 max_krylov),
-                                                    ctl);
+      launch_pdl(k_small_newton, 1, kSmallThreads, 0, im.s, (int)n, gdt, X, RX, S, V[0], krylov_tol,
+                 std::min(m, max_krylov), ctl);
       ++im.launches;
       if (!read_ctl() || hctl->gnorm <= newton_tol * hctl->snorm) break;
       if (it == 20) {
