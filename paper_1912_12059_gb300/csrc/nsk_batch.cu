@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(TPB, (nsk::lift_min_blocks<R, TPB>())) k_bphas
                                                      const int* __restrict__ blk2inst, int* __restrict__ err) {
   constexpr int G4 = nsk::group_for<3, 4>(TPB), G5 = nsk::group_for<3, 5>(TPB);
   constexpr int a = nsk::lift_smem<R, 3, 4, G4>(), c = nsk::lift_smem<R, 3, 5, G5>();
-  __shared__ R sm[a > c ? a : c];
+  __shared__ __align__(16) R sm[a > c ? a : c];
   __shared__ __align__(16) unsigned char spraw[sizeof(NskParams)];
   NskParams* sp = (NskParams*)spraw;
   const int i = blk2inst[blockIdx.x];
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(TPB) k_bphase_volume(const BatchInst* __restri
                                                        const R B, int* __restrict__ err, const int write_traces) {
   constexpr int G4 = nsk::group_for<3, 4>(TPB), G5 = nsk::group_for<3, 5>(TPB);
   constexpr int a = nsk::volume_smem<R, 3, 4, G4, FUSED>(), c = nsk::volume_smem<R, 3, 5, G5, FUSED>();
-  __shared__ R sm[a > c ? a : c];
+  __shared__ __align__(16) R sm[a > c ? a : c];
   __shared__ __align__(16) unsigned char spraw[sizeof(NskParams)];
   NskParams* sp = (NskParams*)spraw;
   const int i = blk2inst[blockIdx.x];
