@@ -48,6 +48,17 @@ int nsk_test_hook_mlp_fwd_kernel(int which);
  * synchronisation. NSK_ERR_ARG for another fn, NULL arrays or n < 0. */
 int nsk_test_hook_math(int fn, const double* x, double* y, long long n, void* stream);
 
+/* The line contractions of the FP64 operator (2D and 3D contexts with N >= 2,
+ * parameters set) on n lines of device doubles, each the doubled -1 face value,
+ * the N + 1 nodal values and the doubled +1 face value, in direction dir (0 to
+ * dim - 1): sums[n][N + 1] the weak-form volume and surface sums (2/h folded
+ * in; times mu with with_mu = 1), ends[n][2] the interpolation of the nodal
+ * values to the -1 and +1 face. Queued on the context's stream, no
+ * synchronisation. NSK_ERR_ARG for other contexts or arguments, NSK_ERR_STATE
+ * before nsk_set_params. */
+int nsk_test_hook_lines(nsk_ctx* ctx, int dir, int with_mu, const double* lines, double* sums, double* ends,
+                        long long n);
+
 /* Bounds-checking build only (libnsk_check.so, compiled with -DNSK_BOUNDS_CHECK):
  * makes the context's neighbour strides point far outside the mesh, so that
  * the index checks of its next stage launches fire: they set the error word's

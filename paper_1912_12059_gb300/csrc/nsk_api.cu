@@ -281,6 +281,19 @@ void fill_fx(NskFx& f, int np, int node_type, const double* rh, double mu) {
   f.el = biased_exp(b.lsum * up);
   for (int j = 0; j < np; ++j) f.l[j] = fx_entry(b.l[j], 1.0, f.el);
   f.mum = (long long)ldexp(frexp(mu, &f.mue), 63);
+  f.lobatto = node_type == NSK_NODES_GAUSS_LOBATTO;
+  // a sum a 2^(e - 2104), 1 <= |a| < 2^62, e the biased exponents of line and table together: normal
+  // FP64 values for 1082 <= e < 3066
+  int e0 = f.el, e1 = f.el;
+  for (int k = 0; k < 3; ++k)
+    if (f.ed[k] > 0)
+      for (const int e : {f.ed[k], f.ed[k] + f.mue}) {
+        e0 = e < e0 ? e : e0;
+        e1 = e > e1 ? e : e1;
+      }
+  const int lo = 1082 - e0 > 100 ? 1082 - e0 : 100, hi = 3066 - e1 < 0x7FF ? 3066 - e1 : 0x7FF;
+  f.lo = (unsigned)(lo < 0x7FF ? lo : 0x7FF) << 20;
+  f.span = hi > lo ? (unsigned)(hi - lo) << 20 : 0;
 }
 
 // index constants of the kernels (after E and ne are known)
@@ -1232,6 +1245,17 @@ int nsk_test_hook_corrupt_neighbours(nsk_ctx* c) {
 #else
   return NSK_ERR_STATE;
 #endif
+}
+
+int nsk_test_hook_lines(nsk_ctx* c, int dir, int with_mu, const double* lines, double* sums, double* ends,
+                        long long n) {
+  if (!c || !lines || !sums || !ends || n < 0 || c->precision != NSK_FP64 || c->dim < 2 || c->np < 3 || dir < 0 ||
+      dir >= c->dim || (with_mu != 0 && with_mu != 1))
+    return NSK_ERR_ARG;
+  if (!c->params_set) return NSK_ERR_STATE;
+  if (n == 0) return NSK_OK;
+  const int r = nsk_launch_lines_hook(c->p, c->np, dir, with_mu, lines, sums, ends, n, c->stream);
+  return r < 0 ? r : NSK_OK;
 }
 
 // ---- checkpoint and resume ----

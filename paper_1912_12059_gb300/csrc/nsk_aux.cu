@@ -163,6 +163,53 @@ extern "C" int nsk_test_hook_math(int fn, const double* x, double* y, long long 
   return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
+// Test hook: the line contractions of the FP64 operator in integers, a line per thread.
+namespace {
+template <int NP>
+__global__ void __launch_bounds__(128) k_lines_hook(const NskParams p, const int k, const int mu, const long long n,
+                                                    const double* x, double* sums, double* ends) {
+  __shared__ __align__(16) int2 tb[nsk::fx_tab_lift_smem<3, NP>() + 1];
+  __shared__ __align__(16) double line[128 * (NP + 2 + (NP & 1))];
+  nsk::fx_stage_tables<3, NP, true>(p.fx, tb);
+  __syncthreads();
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double* g = x + i * (NP + 2);
+    double v[NP];
+    for (int j = 0; j < NP; ++j) v[j] = g[1 + j];
+    // the line with its face values as the kernels keep them: its values, the -1 and the +1 face value
+    double* f = line + threadIdx.x * (NP + 2 + (NP & 1));
+    double* fm = f + NP + (NP & 1);
+    nsk::fx_store<NP>(f, 0, reinterpret_cast<const long long(&)[NP]>(v));
+    fm[0] = g[0];
+    fm[1] = g[NP + 1];
+    long long acc[NP];
+    unsigned m;
+    const int2* t = tb + k * nsk::fx_entries<NP>() + (mu ? nsk::fx_tab_smem<3, NP>() : 0);
+    if (nsk::fx_line<NP>(p, v, fm[1], fm[0], t, acc, m))
+      nsk::fx_keep_line<NP>(p, k, mu != 0, t, acc, m, f, 0, fm, 1);
+    else
+      nsk::fx_plain<NP>(p, k, mu != 0, f, 0, fm, 1);
+    for (int j = 0; j < NP; ++j)
+      sums[i * NP + j] = nsk::fx_value<false>(__double_as_longlong(f[nsk::fx_pos<NP>(0, j)]),
+                                            reinterpret_cast<const int*>(fm)[nsk::fx_word<NP>(p, j, 1)]);
+    nsk::fx_ends<NP>(p, v, p.fx.l, ends[2 * i], ends[2 * i + 1]);
+  }
+}
+}  // namespace
+
+int nsk_launch_lines_hook(const NskParams& p, int np, int k, int mu, const double* x, double* sums, double* ends,
+                          long long n, cudaStream_t s) {
+  const unsigned g = (unsigned)((n + 127) / 128 < 1024 ? (n + 127) / 128 : 1024);
+  switch (np) {
+    case 3: k_lines_hook<3><<<g, 128, 0, s>>>(p, k, mu, n, x, sums, ends); break;
+    case 4: k_lines_hook<4><<<g, 128, 0, s>>>(p, k, mu, n, x, sums, ends); break;
+    case 5: k_lines_hook<5><<<g, 128, 0, s>>>(p, k, mu, n, x, sums, ends); break;
+    case 6: k_lines_hook<6><<<g, 128, 0, s>>>(p, k, mu, n, x, sums, ends); break;
+    default: return NSK_ERR_ARG;
+  }
+  return cudaGetLastError() == cudaSuccess ? 1 : NSK_ERR_CUDA;
+}
+
 // ---- single-block schedule: dispatch by dimension ----
 size_t nsk_block_bytes(int dim, const NskParams& p, int np, bool fp32) {
   switch (dim) {

@@ -52,6 +52,8 @@ struct NskFx {
   int2 l[NSK_MAXNP];
   long long mum;         // mu = mum 2^(mue - 63), 2^62 <= mum < 2^63 (0: mu = 0)
   int ed[3], el, mue;
+  int lobatto;           // the node set holds the faces: l(+-1) are unit vectors
+  unsigned lo, span;     // high words of the largest values a line may have: m - lo < span
 };
 
 // Components of a face trace: the conservative variables, and in FP64 also
@@ -197,6 +199,10 @@ int nsk_launch_dt(const NskParams& p, int dim, int np, bool fp32, const NskBuffe
 int nsk_launch_diag(const NskParams& p, int dim, int np, bool fp32, const NskBuffers& b, cudaStream_t s);
 // precision conversion of nodal arrays (FP32 mode boundary)
 int nsk_launch_convert(const void* src, bool src64, void* dst, bool dst64, long long n, cudaStream_t s);
+
+// test hook (nsk_test_hook_lines)
+int nsk_launch_lines_hook(const NskParams& p, int np, int k, int mu, const double* x, double* sums, double* ends,
+                          long long n, cudaStream_t s);
 
 // Programmatic dependent launch: a kernel launched with launch_pdl is set up while its predecessor in the
 // stream drains and runs pdl_begin before its first global access, which waits until the predecessor has

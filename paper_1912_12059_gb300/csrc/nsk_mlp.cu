@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(G * nsk::Shape<D, NP>::NPE)
 #pragma unroll
         for (int j = 0; j < NP; ++j) x[j] = sc[le * NPE + n0 + j * st];
         double om, op;
-        nsk::fx_ends<NP>(x, p.fx.l, p.fx.el, om, op);
+        nsk::fx_ends<NP>(p, x, p.fx.l, om, op);
         o[(size_t)(2 * k) * p.nfe + fn] = om;
         o[(size_t)(2 * k + 1) * p.nfe + fn] = op;
       }

@@ -131,16 +131,18 @@ __device__ __forceinline__ void lift2_group(const NskParams& p, const double* __
         double x[NP];
         fx_load<NP>(sg, Lg, x);
         long long acc[NP];
-        const unsigned E =
-            fx_line<NP>(x, fm[NFN], *fm, reinterpret_cast<const int2*>(tb) + k * fx_entries<NP>(), acc);
-        fx_store<NP>(sg, Lg, acc);
-        *fm = __hiloint2double(0, fx_exp(E, p.fx.ed[k]));
+        unsigned m;
+        const int2* t = reinterpret_cast<const int2*>(tb) + k * fx_entries<NP>();
+        if (fx_line<NP>(p, x, fm[NFN], *fm, t, acc, m))
+          fx_keep_line<NP>(p, k, false, t, acc, m, sg, Lg, fm, NFN);
+        else
+          fx_plain<NP>(p, k, false, sg, Lg, fm, NFN);
       }
     }
     __syncthreads();
     if (valid) {
       double l1[1];
-      volume_sums_fx<D, NP, 1>(sg, sgs, le, n, l1);
+      volume_sums_fx<D, NP, 1>(p, sg, sgs, le, n, l1);
       lap = -l1[0];
       Q2[g] = lap;
     }
@@ -178,7 +180,7 @@ __device__ __forceinline__ void lift2_group(const NskParams& p, const double* __
           double x[NP];
 #pragma unroll
           for (int j = 0; j < NP; ++j) x[j] = sq[(le * (NQ + 1) + c) * NPE + n0 + j * st];
-          fx_ends<NP>(x, p.fx.l, p.fx.el, tm[c], tp[c]);
+          fx_ends<NP>(p, x, p.fx.l, tm[c], tp[c]);
         }
         const size_t off = (size_t)(2 * k) * p.nfe + (e * NFN + fn);
         double f[D];
@@ -346,7 +348,7 @@ __device__ __forceinline__ void volume_group(const NskParams& p, double* __restr
     __syncthreads();
     if (valid) {
       double res[NV];
-      volume_sums_fx<D, NP, NV>(sf, sfs, le, n, res);
+      volume_sums_fx<D, NP, NV>(p, sf, sfs, le, n, res);
       const double Bdt = B * dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {

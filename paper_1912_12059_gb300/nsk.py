@@ -90,6 +90,8 @@ SIGNATURES = {
     "nsk_test_hook_tc_grid_cap": (C.c_int, [C.c_int]),
     "nsk_test_hook_mlp_fwd_kernel": (C.c_int, [C.c_int]),
     "nsk_test_hook_math": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
+    "nsk_test_hook_lines": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p,
+                                      C.c_longlong]),
     "nsk_test_hook_corrupt_neighbours": (C.c_int, [C.c_void_p]),
     "nsk_batch_destroy": (None, [C.c_void_p]),
     "nsk_gemm_bf16": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
@@ -473,6 +475,17 @@ class Solver:
         if n < 0:
             raise NskError(n, "nsk_get_profile")
         return {self.KERNELS[k]: (ms[k], cnt[k]) for k in range(min(n, nk)) if cnt[k] or k < 4}
+
+    def _test_hook_lines(self, lines, direction=0, with_mu=False):
+        """Test-only (include/nsk_test_hooks.h): the FP64 operator's contractions of the lines [n][N + 3] (a
+        float64 CUDA tensor): (sums [n][N + 1], face values [n][2])."""
+        sums = lines.new_empty((lines.shape[0], self.N + 1))
+        ends = lines.new_empty((lines.shape[0], 2))
+        _check(load_library().nsk_test_hook_lines(self.ctx, int(direction), int(bool(with_mu)),
+                                                  C.c_void_p(lines.data_ptr()), C.c_void_p(sums.data_ptr()),
+                                                  C.c_void_p(ends.data_ptr()), int(lines.shape[0])),
+               "nsk_test_hook_lines")
+        return sums, ends
 
     @property
     def launch_count(self):
