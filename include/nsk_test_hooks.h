@@ -42,11 +42,16 @@ int nsk_test_hook_tc_grid_cap(int max_ctas);
 int nsk_test_hook_mlp_fwd_kernel(int which);
 
 /* The FP64 reciprocal (fn = 0) and square root (fn = 1) the stage kernels use
- * (Newton-Raphson from the FP32 hardware approximations; CUDA's own division
- * and sqrt outside 2^-120 < x < 2^120), evaluated on the device arrays x -> y
+ * (fixed-point Newton steps from the FP32 hardware approximations; CUDA's own
+ * division and sqrt outside 2^-120 < x < 2^120), evaluated on the device arrays x -> y
  * of n values on stream, for their accuracy tests. Queued, no
  * synchronisation. NSK_ERR_ARG for another fn, NULL arrays or n < 0. */
 int nsk_test_hook_math(int fn, const double* x, double* y, long long n, void* stream);
+
+/* The stage kernels' quotients x / y of device arrays (precision NSK_FP32_MIXED:
+ * of the values rounded to FP32), into q. Queued on stream, no synchronisation.
+ * NSK_ERR_ARG for another precision, NULL arrays or n < 0. */
+int nsk_test_hook_div(int precision, const double* x, const double* y, double* q, long long n, void* stream);
 
 /* The line contractions of the FP64 operator (2D and 3D contexts with N >= 2,
  * parameters set) on n lines of device doubles, each the doubled -1 face value,

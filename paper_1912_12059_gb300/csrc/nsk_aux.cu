@@ -163,6 +163,23 @@ extern "C" int nsk_test_hook_math(int fn, const double* x, double* y, long long 
   return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
 }
 
+// Test hook: the quotients of the stage kernels (FP64, or FP32 on the values rounded to FP32).
+namespace {
+__global__ void __launch_bounds__(256) k_div_hook(const int fp32, const double* x, const double* y, double* q,
+                                                  const long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    q[i] = fp32 ? (double)nsk::div_s((float)x[i], (float)y[i]) : nsk::div_s(x[i], y[i]);
+}
+}  // namespace
+
+extern "C" int nsk_test_hook_div(int precision, const double* x, const double* y, double* q, long long n,
+                                 void* stream) {
+  if ((precision != NSK_FP64 && precision != NSK_FP32_MIXED) || !x || !y || !q || n < 0) return NSK_ERR_ARG;
+  if (n == 0) return NSK_OK;
+  k_div_hook<<<reduce_grid(n), 256, 0, (cudaStream_t)stream>>>(precision == NSK_FP32_MIXED, x, y, q, n);
+  return cudaGetLastError() == cudaSuccess ? NSK_OK : NSK_ERR_CUDA;
+}
+
 // Test hook: the line contractions of the FP64 operator in integers, a line per thread.
 namespace {
 template <int NP>

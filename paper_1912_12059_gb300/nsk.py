@@ -90,6 +90,7 @@ SIGNATURES = {
     "nsk_test_hook_tc_grid_cap": (C.c_int, [C.c_int]),
     "nsk_test_hook_mlp_fwd_kernel": (C.c_int, [C.c_int]),
     "nsk_test_hook_math": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
+    "nsk_test_hook_div": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
     "nsk_test_hook_lines": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p,
                                       C.c_longlong]),
     "nsk_test_hook_corrupt_neighbours": (C.c_int, [C.c_void_p]),
@@ -224,6 +225,15 @@ def _test_hook_math(fn, x, y, stream=None):
     _check(load_library().nsk_test_hook_math(int(fn), C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()),
                                              int(x.numel()), C.c_void_p(stream) if stream else None),
            "nsk_test_hook_math")
+
+
+def _test_hook_div(x, y, precision=NSK_FP64, stream=None):
+    """Test-only (include/nsk_test_hooks.h): the stage kernels' quotients of two float64 CUDA tensors."""
+    q = x.new_empty(x.shape)
+    _check(load_library().nsk_test_hook_div(int(precision), C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()),
+                                            C.c_void_p(q.data_ptr()), int(x.numel()),
+                                            C.c_void_p(stream) if stream else None), "nsk_test_hook_div")
+    return q
 
 
 def measure_fma_rate(precision=NSK_FP64, iters=1 << 16, stream=None):
