@@ -1477,9 +1477,18 @@ inline int launch_gemm(const GemmArgs& a, cudaStream_t s) {
                        (!(a.epi == EPI_GELU && a.out) || ((a.ldo % 4) == 0 && a16(a.out))) &&
                        (a.epi != EPI_DGELU || ((a.ldz % 4) == 0 && a16(a.zin)));
   const bool resident = a.epi != EPI_ATOMIC && a.k_split >= a.K && a.K <= 256 && aligned;
+  // an output may lie over A (a hidden layer in place): a block then has to read its rows before any column of them
+  // is written, so all columns stay with one block
+  auto over_a = [&](const void* p, size_t elem, int rows, int ld, int cols) {
+    const uintptr_t a0 = (uintptr_t)a.A, a1 = a0 + 2 * ((size_t)(a.M - 1) * a.lda + a.K);
+    const uintptr_t o0 = (uintptr_t)p, o1 = o0 + elem * ((size_t)(rows - 1) * ld + cols);
+    return p && o0 < a1 && a0 < o1;
+  };
+  const bool in_place = over_a(a.out, 4, a.M, a.ldo, a.N) || over_a(a.hout, 2, a.M, a.ldh, a.N) ||
+                        over_a(a.hout_t, 2, a.N, a.ldt, a.M);
   // few row tiles: 64-column slices fill the SMs (4096 rows of a 256 x 256 layer: 128 blocks instead of
   // 32, each with a quarter of the epilogue); many: one block per SM holds the whole B
-  if (resident && (ntiles * ((a.N + 63) / 64) <= sms || a.N % 64)) {
+  if (resident && !in_place && (ntiles * ((a.N + 63) / 64) <= sms || a.N % 64)) {
     GemmArgs b = a;
     b.nslice = 64;
     while (b.nslice > 16 && ntiles * ((a.N + b.nslice / 2 - 1) / (b.nslice / 2)) <= sms) b.nslice /= 2;
@@ -1488,7 +1497,7 @@ inline int launch_gemm(const GemmArgs& a, cudaStream_t s) {
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
     const int gx = (int)persistent_grid(ntiles, sms / ny > 0 ? sms / ny : 1);
     launch_pdl(k_gemm_tc_rb, dim3((unsigned)gx, (unsigned)ny), kRbThreads, smem, s, b);
-  } else if (resident) {
+  } else if (resident && a.N % 64 == 0) {
     int smem = rb_b_bytes(a.N, a.K) + kBM * a.K * 2 + kRbStageBytes;
     smem = smem < kRbSmemMin ? kRbSmemMin : smem;
     if (smem > kRbSmemMax) return NSK_ERR_ARG;
