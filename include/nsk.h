@@ -319,11 +319,14 @@ int nsk_measure_fma_rate(int precision, int iters, double* tflops, double* ms, v
  * values. */
 int nsk_set_schedule(nsk_ctx* ctx, int tpb, int fused_face);
 int nsk_get_schedule(nsk_ctx* ctx, int* tpb, int* fused_face);
-/* Autotuner: times one residual evaluation under each schedule (tpb 128 and
+/* Autotuner: times the stages of a step under each schedule (tpb 128 and
  * 256 with fused_face 0, 1, 2, and 3 and 4 where they apply; fused_face 0 and 1 for
  * the original NSK equations) on the context's current state (the state is not
  * modified), keeps the fastest and returns it (any output may be NULL; ms_out =
- * its time). */
+ * its time a stage). When that is the single-block schedule (3), it is used where
+ * a call's steps run in its one launch; adaptive and learned-closure steps, the
+ * implicit steps and residuals take the fastest schedule of several launches
+ * (a residual the single-block launch where that is faster for one). */
 int nsk_autotune(nsk_ctx* ctx, int* tpb_out, int* fused_out, double* ms_out);
 
 /* Batched execution (many instances per launch). A batch groups n existing

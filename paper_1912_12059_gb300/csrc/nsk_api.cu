@@ -6,6 +6,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <mutex>
@@ -424,9 +425,11 @@ bool line_eligible(const nsk_ctx* c) {
 }
 
 int launch_stage(nsk_ctx* c, NskLaunch l) {
-  if (l.fused_face == 3) {  // single-block schedule: a residual in one launch; otherwise the separate face pass
-    if (l.mode == NSK_MODE_RHS && block_eligible(c)) return launch_block(c, 1, 0.0, l.Rout);
-    l.fused_face = 0;
+  if (l.fused_face == 3) {  // single-block schedule: a residual in one launch; otherwise several
+    if (l.mode == NSK_MODE_RHS && (!c->ml_tpb || c->block_rhs) && block_eligible(c))
+      return launch_block(c, 1, 0.0, l.Rout);
+    l.tpb = c->multi_tpb();
+    l.fused_face = c->multi_fused();
   }
   // kernels 0..3 = prolong, lift, face, volume
   const int mask = c->p.model == NSK_MODEL_NSK ? (l.mode == NSK_MODE_LIFT ? 3 : 15)
@@ -844,9 +847,10 @@ int nsk_step(nsk_ctx* c, double dt, int nsteps) {
         const int r = nsk_closure_apply_ctx(c, ready ? c->b.Utr : nullptr);
         if (r) return r;
       }
-      // (the single-block schedule, where it does not apply, steps with the separate face pass)
-      const int ff = c->fused_face == 3 ? 0 : c->fused_face;
-      NskLaunch l = {NSK_MODE_LSRK, nullptr, kA[st], kB[st], adaptive ? c->b.dt : nullptr, dt, nullptr, c->tpb, ff};
+      // (where the single-block schedule does not apply, the tuned schedule of several launches)
+      const int ff = c->multi_fused();
+      NskLaunch l = {NSK_MODE_LSRK, nullptr, kA[st], kB[st], adaptive ? c->b.dt : nullptr, dt, nullptr,
+                     c->multi_tpb(), ff};
       // the volume kernel writes the traces of the updated state for the next stage of this call
       const bool write = c->p.model != NSK_MODEL_NSK && !(s == nsteps - 1 && st == 4);
       l.traces_ready = ready;
@@ -1140,6 +1144,7 @@ int nsk_set_schedule(nsk_ctx* c, int tpb, int fused_face) {
   if (!c || (tpb != 128 && tpb != 256) || fused_face < 0 || fused_face > 4) return NSK_ERR_ARG;
   c->tpb = tpb;
   c->fused_face = fused_face;
+  c->ml_tpb = 0;
   return NSK_OK;
 }
 
@@ -1157,8 +1162,9 @@ int nsk_autotune(nsk_ctx* c, int* tpb_out, int* fused_out, double* ms_out) {
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return NSK_ERR_CUDA;
   const int tpbs[2] = {128, 256};
-  double best = 1e300;
+  double best = 1e300, block = 1e300;
   int bt = c->tpb, bf = c->fused_face, st = NSK_OK;
+  bool block_rhs = false;
   const bool prof = c->prof_on;
   c->prof_on = false;
   // the lean two-launch stage applies to relaxation model II only (the original NSK equations
@@ -1168,8 +1174,17 @@ int nsk_autotune(nsk_ctx* c, int* tpb_out, int* fused_out, double* ms_out) {
   sched[nsched++] = 0;
   sched[nsched++] = 1;
   if (c->p.model != NSK_MODEL_NSK) sched[nsched++] = 2;
-  if (c->p.model != NSK_MODEL_NSK && block_eligible(c)) sched[nsched++] = 3;
   if (line_eligible(c)) sched[nsched++] = 4;
+  // device time of reps launches by f, ms each
+  auto timed = [&](int reps, auto&& f) {
+    cudaEventRecord(e0, c->stream);
+    for (int r = 0; r < reps && st == NSK_OK; ++r) st = f();
+    cudaEventRecord(e1, c->stream);
+    if (cudaEventSynchronize(e1) != cudaSuccess) st = NSK_ERR_CUDA;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    return st == NSK_OK ? ms / (double)reps : 1e300;
+  };
   for (int it = 0; it < 2 && st == NSK_OK; ++it)
     for (int f = 0; f < nsched && st == NSK_OK; ++f) {
       c->tpb = tpbs[it];
@@ -1181,30 +1196,39 @@ int nsk_autotune(nsk_ctx* c, int* tpb_out, int* fused_out, double* ms_out) {
       // volume kernel (to the spare buffer: U does not change in RHS mode)
       l.traces_ready = 1;
       l.utr_next = c->utr_alt;
-      // (the single-block schedule runs a step's five stages in one launch: a launch per residual, 13.2 us
-      // with 64 1D elements, would lose to separate kernels at 11.8, which overlap their launches and
-      // take 14.8 a stage in a step against its 10.2)
-      const int reps = sched[f] == 3 ? 5 : 3;
-      cudaEventRecord(e0, c->stream);
-      if (sched[f] == 3)
-        st = launch_block(c, reps, 0.0, c->rbuf);
-      else
-        for (int r = 0; r < reps && st == NSK_OK; ++r) st = launch_stage(c, l);
-      cudaEventRecord(e1, c->stream);
-      if (cudaEventSynchronize(e1) != cudaSuccess) st = NSK_ERR_CUDA;
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (st == NSK_OK && ms / reps < best) {
-        best = ms / reps;
+      const double ms = timed(3, [&] { return launch_stage(c, l); });
+      if (ms < best) {
+        best = ms;
         bt = c->tpb;
         bf = c->fused_face;
       }
     }
+  // The single-block schedule takes a fixed-dt step's five stages in one launch and is timed so; a residual
+  // alone takes a launch of its own and competes as one with the fastest of the others (with its prolongation
+  // pass, as a call makes it). 64 1D elements, N = 3: 10.2 us a stage in a step against 14.8, 13.2 a residual
+  // alone against 11.8.
+  if (st == NSK_OK && c->p.model != NSK_MODEL_NSK && block_eligible(c)) {
+    block = timed(1, [&] { return launch_block(c, 5, 0.0, c->rbuf); });
+    block = std::min(block, timed(1, [&] { return launch_block(c, 5, 0.0, c->rbuf); })) / 5.0;
+    NskLaunch l = {NSK_MODE_RHS, c->rbuf, 0.0, 0.0, nullptr, 0.0, nullptr, bt, bf};
+    const double one = timed(5, [&] { return launch_block(c, 1, 0.0, c->rbuf); });
+    const double sep = timed(5, [&] { return launch_stage(c, l); });
+    block_rhs = one < sep;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->prof_on = prof;
   c->tpb = bt;
   c->fused_face = bf;
+  c->ml_tpb = 0;
+  if (block < best) {
+    c->fused_face = 3;
+    c->ml_tpb = bt;
+    c->ml_fused = bf;
+    c->block_rhs = block_rhs;
+    bf = 3;
+    best = block;
+  }
   if (st) return st;
   if (tpb_out) *tpb_out = bt;
   if (fused_out) *fused_out = bf;

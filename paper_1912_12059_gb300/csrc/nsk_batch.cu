@@ -483,12 +483,15 @@ cudaStream_t inst_stream(const nsk_batch* bt, int i) { return bt->naux < 2 ? bt-
 // instance schedule: one stage of instance i by its own stage kernels, on stream i mod naux.
 // fused 5: each instance's own schedule (its tpb and fused_face; the lean and single-block schedules
 // run as the separate face pass there)
-int inst_fused(const nsk_ctx* c) { return (c->fused_face == 1 || c->fused_face == 4) ? c->fused_face : 0; }
+int inst_fused(const nsk_ctx* c) {
+  const int f = c->multi_fused();
+  return (f == 1 || f == 4) ? f : 0;
+}
 int launch_instance(nsk_batch* bt, int i, int mode, double A, double B, int tpb, int fused, int traces) {
   nsk_ctx* c = bt->inst[i];
   const int fi = fused == 5 ? inst_fused(c) : fused;
   const int tr = fi == 1 ? 0 : traces;  // the fused volume phase prolongs every stage
-  NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, fused == 5 ? c->tpb : tpb, fi};
+  NskLaunch l = {mode, c->rbuf, A, B, c->b.dt, 0.0, nullptr, fused == 5 ? c->multi_tpb() : tpb, fi};
   l.traces_ready = tr & 1;
   l.utr_next = (tr & 2) ? c->b.Utr : nullptr;  // separate face schedule: written in place
   const int r = nsk_launch_stage_d3(c->p, c->np, c->precision == NSK_FP32_MIXED, c->b, l, inst_stream(bt, i));
@@ -519,7 +522,7 @@ int launch_instance_lean(nsk_batch* bt, int i, int mode, double A, double B, int
 unsigned long long inst_schedules(const nsk_batch* bt) {
   unsigned long long h = 1469598103934665603ull;  // FNV-1a over the pairs
   for (const nsk_ctx* c : bt->inst) {
-    h = (h ^ (unsigned long long)(c->tpb == 128 ? 1 : 2)) * 1099511628211ull;
+    h = (h ^ (unsigned long long)(c->multi_tpb() == 128 ? 1 : 2)) * 1099511628211ull;
     h = (h ^ (unsigned long long)inst_fused(c)) * 1099511628211ull;
   }
   return h;

@@ -280,6 +280,13 @@ struct nsk_ctx {
   double prof_ms[NSK_NKERN];
   long long prof_cnt[NSK_NKERN];
   int tpb, fused_face;  // stage schedule (nsk_set_schedule / nsk_autotune)
+  // beside a tuned single-block schedule (fused_face 3): the fastest schedule of several launches, for the
+  // calls that cannot take a step in one (ml_tpb 0: none, set by hand), and whether a residual alone is
+  // faster in one launch too
+  int ml_tpb, ml_fused;
+  bool block_rhs;
+  int multi_tpb() const { return fused_face == 3 && ml_tpb ? ml_tpb : tpb; }
+  int multi_fused() const { return fused_face == 3 ? (ml_tpb ? ml_fused : 0) : fused_face; }
   // learned c-closure (nsk_set_closure)
   int closure_mode;            // NSK_C_EXPLICIT or NSK_C_LEARNED
   struct nsk_mlp* mlp;         // borrowed network
