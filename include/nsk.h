@@ -311,7 +311,8 @@ int nsk_measure_fma_rate(int precision, int iters, double* tflops, double* ms, v
  *     and stores, contractions along the line in registers); elsewhere the
  *     separate face pass runs.
  * Default: tpb 256, separate face pass. (FP64 elements in 2D and 3D with
- * N >= 3 always run 128-thread blocks: faster at every size measured.) Every expression that could be
+ * N >= 3 always run 128-thread blocks under 0 and 1: faster at every size
+ * measured; the autotuner reports them as 128.) Every expression that could be
  * contracted into a fused multiply-add in more than one way is written as an
  * explicit fma (and the FP64 line contractions in 2D and 3D with N >= 2 are exact integer sums,
  * rounded once), and every schedule evaluates each value with the same code,

@@ -1185,8 +1185,12 @@ int nsk_autotune(nsk_ctx* c, int* tpb_out, int* fused_out, double* ms_out) {
     cudaEventElapsedTime(&ms, e0, e1);
     return st == NSK_OK ? ms / (double)reps : 1e300;
   };
+  // FP64 elements with N >= 3 in 2D and 3D run 128-thread blocks under schedules 0 and 1 whatever tpb says
+  // (small_blocks): one candidate each, reported as what runs
+  const bool small = c->precision == NSK_FP64 && c->dim >= 2 && c->np >= 4 && c->p.model != NSK_MODEL_NSK;
   for (int it = 0; it < 2 && st == NSK_OK; ++it)
     for (int f = 0; f < nsched && st == NSK_OK; ++f) {
+      if (small && it == 1 && sched[f] < 2) continue;
       c->tpb = tpbs[it];
       c->fused_face = sched[f];
       NskLaunch l = {NSK_MODE_RHS, c->rbuf, 0.0, 0.0, nullptr, 0.0, nullptr, c->tpb, c->fused_face};

@@ -90,3 +90,14 @@ def test_schedules_set_by_hand_stay(gpu):
     assert s.get_profile()["k_block"][1] == 1
     assert s.get_schedule() == (256, 3)
     s.close()
+
+
+@pytest.mark.parametrize("dim,ne,N", [(2, (24, 24), 3), (3, (6, 6, 6), 4)])
+def test_tuner_reports_the_blocks_that_run(gpu, dim, ne, N):
+    """FP64, N >= 3, 2D and 3D: schedules 0 and 1 run 128-thread blocks, so that is what the tuner reports."""
+    s, _ = _solver(dim, ne, N)
+    for _ in range(12):
+        s.set_schedule(256, 0)
+        tpb, fused, _ = s.autotune()
+        assert fused not in (0, 1) or tpb == 128
+    s.close()
