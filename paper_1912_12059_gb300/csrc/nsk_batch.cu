@@ -535,19 +535,23 @@ unsigned long long inst_schedules(const nsk_batch* bt) {
 // (the line schedule, fused_face 4, is a separate face schedule)
 int step_traces(int fused) { return (fused == 0 || fused == 4 || fused == 5) ? 3 : 0; }
 
-// stamps: the last stage of a step whose per-instance latencies are measured (each instance's
-// completion stamped after its last kernel; one launch for all instances stamps them together)
+// `stages` residuals of every instance under the instance schedule, forked onto the auxiliary streams and joined once
+// (lean: each as the given stage of a step, -1 one of its own)
+int launch_instances_rhs(nsk_batch* bt, int tpb, int fused, int traces, int stage, int stages) {
+  int r = fork_aux(bt);
+  if (r) return r;
+  for (int i = 0; i < bt->n; ++i)
+    for (int q = 0; q < stages && r >= 0; ++q)
+      r = fused == 2 ? launch_instance_lean(bt, i, NSK_MODE_RHS, 0.0, 0.0, tpb, stage)
+                     : launch_instance(bt, i, NSK_MODE_RHS, 0.0, 0.0, tpb, fused, fused == 1 ? 0 : traces);
+  const int j = join_aux(bt);
+  return r < 0 ? r : j;
+}
+
+// one stage of all instances in the single-launch schedules; stamps: the last stage of a step whose per-instance
+// latencies are measured (one launch stamps all completions together)
 int launch_batch(nsk_batch* bt, int mode, double A, double B, int tpb, int fused, int persistent, int traces,
-                 bool stamps = false, int stage = -1) {
-  if (persistent == 2) {  // the instance schedule, forked onto the auxiliary streams
-    int r = fork_aux(bt);
-    if (r) return r;
-    for (int i = 0; i < bt->n && r >= 0; ++i)
-      r = fused == 2 ? launch_instance_lean(bt, i, mode, A, B, tpb, stage)
-                     : launch_instance(bt, i, mode, A, B, tpb, fused, fused == 1 ? 0 : traces);
-    const int j = join_aux(bt);
-    return r < 0 ? r : j;
-  }
+                 bool stamps = false) {
   if (fused == 1) traces = 0;  // the fused volume phase reads the traces: they are prolonged every stage
   const int r = persistent ? launch_persistent(bt, mode, A, B, tpb, fused, traces)
                            : launch_phases(bt, mode, A, B, tpb, fused, traces);
@@ -777,17 +781,24 @@ int nsk_batch_autotune(nsk_batch* bt, int* tpb_out, int* fused_out, int* persist
         // step runs it (rewriting the traces of the unchanged state leaves them as they are; the
         // lean stage as a middle stage of a step: traces read from the trace buffer, the next
         // ones written to the spare buffer)
-        st = launch_batch(bt, NSK_MODE_RHS, 0.0, 0.0, tpbs[ti], f, per, 0);
+        // (the instance schedule forks and joins its streams once a step of five stages: an instance does not wait for
+        // the slowest one after every stage)
+        const int reps = per == 2 ? 5 : 3;
+        st = per == 2 ? launch_instances_rhs(bt, tpbs[ti], f, 0, -1, 1)
+                      : launch_batch(bt, NSK_MODE_RHS, 0.0, 0.0, tpbs[ti], f, per, 0);
         if (st) break;
         cudaEventRecord(e0, bt->stream);
-        for (int r = 0; r < 3 && st == NSK_OK; ++r)
-          st = launch_batch(bt, NSK_MODE_RHS, 0.0, 0.0, tpbs[ti], f, per, step_traces(f), false, 2);
+        if (per == 2)
+          st = launch_instances_rhs(bt, tpbs[ti], f, step_traces(f), 2, reps);
+        else
+          for (int r = 0; r < reps && st == NSK_OK; ++r)
+            st = launch_batch(bt, NSK_MODE_RHS, 0.0, 0.0, tpbs[ti], f, per, step_traces(f));
         cudaEventRecord(e1, bt->stream);
         if (cudaEventSynchronize(e1) != cudaSuccess) st = NSK_ERR_CUDA;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (st == NSK_OK && ms / 3.0 < best) {
-          best = ms / 3.0;
+        if (st == NSK_OK && ms / reps < best) {
+          best = ms / reps;
           bt_tpb = tpbs[ti];
           bt_f = f;
           bt_p = per;
