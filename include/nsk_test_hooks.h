@@ -64,6 +64,12 @@ int nsk_test_hook_div(int precision, const double* x, const double* y, double* q
 int nsk_test_hook_lines(nsk_ctx* ctx, int dir, int with_mu, const double* lines, double* sums, double* ends,
                         long long n);
 
+/* on = 1: the launches of the implicit integrator's Arnoldi steps report an error
+ * while they are captured into a graph (nsk_step_esdirk), so that it launches
+ * them directly; 0 (the default): no such error. Process-wide; results are the
+ * same. NSK_ERR_ARG for another value. */
+int nsk_test_hook_esdirk_refuse_capture(int on);
+
 /* Bounds-checking build only (libnsk_check.so, compiled with -DNSK_BOUNDS_CHECK):
  * makes the context's neighbour strides point far outside the mesh, so that
  * the index checks of its next stage launches fire: they set the error word's

@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <vector>
 
 #include "nsk_internal.h"
@@ -642,6 +643,8 @@ const double kA6[6][5] = {
     {82889.0 / 524892.0, 0.0, 15625.0 / 83664.0, 69875.0 / 102672.0, -2260.0 / 8211.0},
 };
 
+std::atomic<int> g_refuse_capture{0};  // test hook: an Arnoldi step's launches report an error while captured
+
 struct Implicit {
   nsk_ctx* c;
   long long n;          // values of a state vector
@@ -718,6 +721,12 @@ static int fd_colours(int ne) {
   for (int K = 3; K <= ne; ++K)
     if (ne % K == 0) return K;
   return ne;
+}
+
+extern "C" int nsk_test_hook_esdirk_refuse_capture(int on) {
+  if (on != 0 && on != 1) return NSK_ERR_ARG;
+  g_refuse_capture = on;
+  return NSK_OK;
 }
 
 int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double krylov_tol, int krylov_dim,
@@ -885,6 +894,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
       bool ok = cudaStreamBeginCapture(im.s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
         steps();
+        if (g_refuse_capture) im.status = NSK_ERR_CUDA;
         ok = cudaStreamEndCapture(im.s, &g) == cudaSuccess && g && im.status == NSK_OK &&
              cudaGraphInstantiate(&gchunk, g, 0) == cudaSuccess;
         if (g) cudaGraphDestroy(g);
@@ -896,6 +906,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
         cudaGetLastError();
         gchunk = nullptr;
         graphs = false;
+        im.status = NSK_OK;  // an error of the capture: the direct launches report their own
       }
     }
     if (!graphs) {
@@ -1034,6 +1045,7 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
                 im.status = NSK_ERR_CUDA;
               } else {
                 arnoldi(k);
+                if (g_refuse_capture) im.status = NSK_ERR_CUDA;
                 if (cudaStreamEndCapture(im.s, &g) != cudaSuccess || !g ||
                     cudaGraphInstantiate(&gstep[(size_t)k], g, 0) != cudaSuccess)
                   im.status = NSK_ERR_CUDA;

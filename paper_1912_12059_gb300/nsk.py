@@ -91,6 +91,7 @@ SIGNATURES = {
     "nsk_test_hook_mlp_fwd_kernel": (C.c_int, [C.c_int]),
     "nsk_test_hook_math": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
     "nsk_test_hook_div": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
+    "nsk_test_hook_esdirk_refuse_capture": (C.c_int, [C.c_int]),
     "nsk_test_hook_lines": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p,
                                       C.c_longlong]),
     "nsk_test_hook_corrupt_neighbours": (C.c_int, [C.c_void_p]),
@@ -225,6 +226,11 @@ def _test_hook_math(fn, x, y, stream=None):
     _check(load_library().nsk_test_hook_math(int(fn), C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()),
                                              int(x.numel()), C.c_void_p(stream) if stream else None),
            "nsk_test_hook_math")
+
+
+def _test_hook_esdirk_refuse_capture(on):
+    """Test-only (include/nsk_test_hooks.h): fail the capture of the implicit integrator's Arnoldi steps."""
+    _check(load_library().nsk_test_hook_esdirk_refuse_capture(int(bool(on))), "nsk_test_hook_esdirk_refuse_capture")
 
 
 def _test_hook_div(x, y, precision=NSK_FP64, stream=None):
