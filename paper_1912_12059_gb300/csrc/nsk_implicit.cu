@@ -1031,7 +1031,6 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
               im.stop = &ctl->stop;
               im.c0p = &ctl->c0;
               arnoldi(k);
-              ++im.rhs_evals;
               im.stop = nullptr;
               im.c0p = nullptr;
               return;
@@ -1067,7 +1066,6 @@ int nsk_step_esdirk(nsk_ctx* c, double dt, int nsteps, double newton_tol, double
                 im.stop = &ctl->stop;
                 im.c0p = &ctl->c0;
                 arnoldi(k);
-                ++im.rhs_evals;
                 im.stop = nullptr;
                 im.c0p = nullptr;
                 return;

@@ -36,3 +36,9 @@ def test_refused_capture_falls_back_to_launches(gpu, ne, precond):
     (a, sa), (b, sb) = _both(ne, precond)
     assert np.array_equal(a, b)
     assert all(sa[k] == sb[k] for k in ("newton", "krylov", "failed")) and sa["krylov"] > 4
+
+
+@pytest.mark.parametrize("ne,precond", CASES)
+def test_direct_launches_count_their_residuals_once(gpu, ne, precond):
+    (_, sa), (_, sb) = _both(ne, precond)
+    assert sa["rhs"] == sb["rhs"]
