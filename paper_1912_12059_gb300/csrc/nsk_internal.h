@@ -240,7 +240,7 @@ struct FvBuffers {
   double* Gf;    // [E][2][2] (v_x, c_x) of each element side of its faces
   double* SL;    // [E][N+1][3] MinMod slopes of the FV elements
   double* Fh;    // [E+1][3] element-face fluxes
-  unsigned* bar; // [2] grid barrier of the cooperative small-mesh launch (arrivals, generation)
+  unsigned* bar; // [2] grid barrier of the cooperative small-mesh launch: one 64-bit arrival counter
 };
 int nsk_fv_launch_stage(const NskParams& p, const void* fvp, int np, const FvBuffers& fb, const NskBuffers& b,
                         int mode, double* Rout, double A, double B, const double* dtp, double dtv, cudaStream_t s);
