@@ -881,7 +881,7 @@ namespace {
 // the overlapped path applies: FP64 relaxation model without closure or sub-cells, 3D, N = 3,
 // the separate face pass, no profiling, and NSK_IO_SLABS z-slabs of whole blocks of every
 // stage kernel (each slab whole z planes, a multiple of the 16 elements of a 256-thread
-// prolongation or face-pass block; the lifting and volume blocks hold 2 or 4 elements)
+// prolongation or face-pass block; the lifting and volume blocks hold 2 elements)
 bool host_overlap_eligible(const nsk_ctx* c) {
   if (c->precision != NSK_FP64 || c->dim != 3 || c->np != 4 || c->p.model == NSK_MODEL_NSK || c->fv_path() ||
       c->closure_mode == NSK_C_LEARNED || c->fused_face != 0 || (c->tpb != 128 && c->tpb != 256) || c->prof_on)

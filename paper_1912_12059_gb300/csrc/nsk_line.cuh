@@ -523,23 +523,22 @@ int launch_stage_line(const NskParams& p, const NskBuffers& b, const NskLaunch& 
   const unsigned eb = (unsigned)((p.E + G - 1) / G);
   if (l.mode == NSK_MODE_LIFT) {
     constexpr int GN = group_for<3, 4>(256);
-    launch_pdl(k_lift<float, 3, 4, GN, false>, (unsigned)((p.E + GN - 1) / GN), GN * 64, 0, s,
-        p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q, (float*)b.FVtr, b.err, 0);
+    launch_pdl(k_lift<float, 3, 4, GN, false>, (unsigned)((p.E + GN - 1) / GN), GN * 64, 0, s, p, (const float*)b.U,
+               (const float*)b.Utr, (float*)b.Q, (float*)b.FVtr, b.err, 0);
   } else {
     launch_pdl(k_lift_line<G>, eb, G * 16, smem_lift, s, p, (const float*)b.U, (const float*)b.Utr, (float*)b.Q,
-                                                 (float*)b.FVtr, b.err);
+               (float*)b.FVtr, b.err);
   }
   if (l.ev) cudaEventRecord(l.ev[2], s);
   ++nl;
   if (l.mode != NSK_MODE_LIFT) {
     launch_pdl(k_face<float, 3, 4>, dim3(grid_for(p.nfe, 256), 3), 256, 0, s, p, (const float*)b.Utr,
-               (const float*)b.FVtr,
-                                                                       (float*)b.Fstar, b.err, 0);
+               (const float*)b.FVtr, (float*)b.Fstar, b.err, 0);
     ++nl;
     if (l.ev) cudaEventRecord(l.ev[3], s);
     launch_pdl(k_volume_line<G>, eb, G * 16, smem_vol, s, p, (float*)b.U, (const float*)b.Q, (const float*)b.Fstar,
-                                                  (float*)b.K, (float*)l.Rout, l.mode, (float)l.A, (float)l.B,
-                                                  l.dt_dev, (float)l.dt_val, b.err, (float*)l.utr_next);
+               (float*)b.K, (float*)l.Rout, l.mode, (float)l.A, (float)l.B, l.dt_dev, (float)l.dt_val, b.err,
+               (float*)l.utr_next);
     if (l.ev) cudaEventRecord(l.ev[4], s);
     ++nl;
   }

@@ -420,9 +420,8 @@ int nsk_mlp_train_step(nsk_mlp* m, const void* X, const float* T, int batch, dou
   const float c1 = 1.0f - powf(b1, (float)m->adam_step), c2 = 1.0f - powf(b2, (float)m->adam_step);
   AdamLayers L = {{m->W1, m->W2, m->W3}, {m->W1t, m->W2t, m->W3t}, {(int)m->oW1, (int)m->oW2, (int)m->oW3},
                   {m->h1, m->h2, m->nout}, {m->nin_pad, m->h1, m->h2}};
-  launch_pdl(k_adam, nb((long long)m->nparam), 256, 0, m->stream, m->param, m->grad, m->m1, m->m2, (int)m->nparam,
-             (float)lr,
-                                                          b1, b2, 1e-8f, c1, c2, L);
+  launch_pdl(k_adam,
+             nb((long long)m->nparam), 256, 0, m->stream, m->param, m->grad, m->m1, m->m2, (int)m->nparam, (float)lr, b1, b2, 1e-8f, c1, c2, L);
   m->launches += 1;
   if (cudaGetLastError() != cudaSuccess) return NSK_ERR_CUDA;
   return loss ? mlp_check(m, loss, batch) : NSK_OK;

@@ -542,24 +542,21 @@ int launch_stage_g(const NskParams& p, const NskBuffers& b, const NskLaunch& l, 
   if (l.ev) cudaEventRecord(l.ev[1], s);
   const unsigned eb = (unsigned)((p.E + G - 1) / G);
   launch_pdl(k_lift_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (const double*)b.U, (const double*)b.Utr, (double*)b.Q,
-                                                  (double*)b.Gtr, b.err);
+             (double*)b.Gtr, b.err);
   ++nl;
   if (l.mode != NSK_MODE_LIFT) {
     launch_pdl(k_lift2_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (const double*)b.U, (const double*)b.Utr,
-                                                     (const double*)b.Q, (const double*)b.Gtr, (double*)b.Q2,
-                                                     (double*)b.FVtr);
+               (const double*)b.Q, (const double*)b.Gtr, (double*)b.Q2, (double*)b.FVtr);
     ++nl;
   }
   if (l.ev) cudaEventRecord(l.ev[2], s);
   if (l.mode != NSK_MODE_LIFT) {
     launch_pdl(k_face_nsk<D, NP>, dim3(grid_for(p.nfe, 256), D), 256, 0, s, p, (const double*)b.Utr,
-               (const double*)b.FVtr,
-                                                                     (double*)b.Fstar, b.err);
+               (const double*)b.FVtr, (double*)b.Fstar, b.err);
     ++nl;
     if (l.ev) cudaEventRecord(l.ev[3], s);
     launch_pdl(k_volume_nsk<D, NP, G>, eb, G * S::NPE, 0, s, p, (double*)b.U, (const double*)b.Q, (const double*)b.Q2,
-                                                      (const double*)b.Fstar, (double*)b.K, (double*)l.Rout, l.mode,
-                                                      l.A, l.B, l.dt_dev, l.dt_val, b.err);
+               (const double*)b.Fstar, (double*)b.K, (double*)l.Rout, l.mode, l.A, l.B, l.dt_dev, l.dt_val, b.err);
     ++nl;
     if (l.ev) cudaEventRecord(l.ev[4], s);
   }
