@@ -867,6 +867,12 @@ def measure_coalescence2d_variant(args, stream, peaks):
     return out
 
 
+def solo_schedule(s, tpb, fused):
+    """Give an instance stepped alone the batch's schedule (5: its own, which the batch's tuner has set)."""
+    if fused != 5:
+        s.set_schedule(tpb, fused)
+
+
 def measure_batch_variant(args, n=32, steps=None, with_sequential=True):
     """Batched serving of n uneven 3D collision instances (16^3..48^3 elements, N in {3, 4}, We and
     impact parameter drawn per instance), FP32 operator, autotuned schedule, CUDA-graph replay:
@@ -911,7 +917,7 @@ def measure_batch_variant(args, n=32, steps=None, with_sequential=True):
     if with_sequential:  # the same instances stepped one after another (no batching)
         seq_ms = 0.0
         for s in solvers:
-            s.set_schedule(tpb, fused)
+            solo_schedule(s, tpb, fused)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             torch.cuda.synchronize()
             e0.record()

@@ -552,7 +552,7 @@ class Batch:
         return t.value, f.value, p.value
 
     def autotune(self):
-        """Time all ten schedules on the batch; keep and return (tpb, fused, persistent, ms)."""
+        """Time the schedules on the batch; keep the fastest and return its (tpb, fused, persistent, ms a stage)."""
         t, f, p, ms = C.c_int(), C.c_int(), C.c_int(), C.c_double()
         _check(load_library().nsk_batch_autotune(self.h, C.byref(t), C.byref(f), C.byref(p), C.byref(ms)),
                "nsk_batch_autotune")
