@@ -439,7 +439,9 @@ def run_gpu(args, wl, rank, world):
         roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                 "traffic": traffic, "kernel": name, "peak_source": hbm_src,
                 "algorithmic_per_launch": bytes_e * s.E}
-        if prec == nsk.NSK_FP64:
+        if prec == nsk.NSK_FP64:  # bound by the integer and FP64 pipes; the fraction is of the copy bandwidth
+            roof["bound"] = "alu"
+            roof["frac_of"] = "hbm"
             roof["probe_fp64_tflops"] = probe64
             roof["probe_sm_mhz_median"] = probe_clk
     roof["traffic_source"] = TRAFFIC_SOURCE if traffic is not None else None

@@ -315,7 +315,7 @@ int nsk_measure_fma_rate(int precision, int iters, double* tflops, double* ms, v
  * measured; the autotuner reports them as 128.) Every expression that could be
  * contracted into a fused multiply-add in more than one way is written as an
  * explicit fma (and the FP64 line contractions in 2D and 3D with N >= 2 are exact integer sums,
- * rounded once), and every schedule evaluates each value with the same code,
+ * rounded once, or for rare lines FP64 sums of one order), and every schedule evaluates each value with the same code,
  * so results are bit-identical under every schedule. NSK_ERR_ARG for other
  * values. */
 int nsk_set_schedule(nsk_ctx* ctx, int tpb, int fused_face);
@@ -398,6 +398,7 @@ void nsk_batch_destroy(nsk_batch* batch);
  *   and, if hout_t is not NULL, its transpose -> hout_t (BF16 [N][ldt]);
  * 3 dz = C * GELU'(zin[M][ldz]) -> hout (BF16) and hout_t, column sums of dz
  *   added to bias_grad (if not NULL).
+ * The output may lie over A's rows (a hidden layer in place).
  * GELU(x) = x Phi(x) (exact, with erf). err: device int that receives
  * NSK_EBIT_TIMEOUT (8) if a bounded tensor-core wait expires (NULL: an
  * internal word). Queued on stream; no synchronisation. No counterpart in the

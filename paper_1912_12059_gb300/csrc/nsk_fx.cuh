@@ -25,9 +25,9 @@
 // row (fx_leaves). A line whose largest value lies outside the range in which sums neither overflow nor lose bits
 // below 2^-1022 (NskFx; infinities, NaN and tiny values among them) takes FP64 sums and hands them on as they are.
 //
-// Measured (64^3 elements, N = 3, ms a stage, FP64 sums before): lifting 3.77 -> 1.44, volume 5.15 ->
-// 1.80, prolongation 1.35 -> 0.56 (without the provisions for zero entries and for the range: 1.45, 1.73, 0.56). Bound now: the lifting by integer issue (ALU pipe 68 %, issue slots
-// 62 %, FP64 32 %), the volume kernel by both pipes (FP64 66 %, ALU 64 %) at 3.1 TB/s of DRAM traffic.
+// Measured (64^3 elements, N = 3, ms a stage, FP64 sums before): lifting 3.77 -> 1.42, volume 5.15 ->
+// 1.82, prolongation 1.35 -> 0.56 (without the provisions for zero entries and for the range: 1.43, 1.73, 0.56). Bound now: the lifting by integer issue (ALU pipe 68 %, issue slots
+// 67 %, FP64 33 %), the volume kernel by both pipes (FP64 63 %, ALU 62 %) at 3.0 TB/s of DRAM traffic.
 //
 // Bounds: |h| <= 2^30, pair sums and differences in [-2^31, 2^31 - 1] and their low limbs below 2^29 in
 // magnitude, row sums of |matrix h| <= 2^30, at most 4 terms a product sum: |sum h h| <= 2^61,
